@@ -5,22 +5,20 @@
 
 #include <cuda_runtime.h>
 
+#include "df.cuh"
+
 namespace sps {
 
-// FP64, for the once-per-galaxy set-up (zero points, lambda_eff, c_SSP).
-__device__ __forceinline__ double tab_T64(const double* __restrict__ T, int n, double u) {
-    if (!(u >= 0.0 && u <= (double)(n - 1))) return 0.0;
-    const int m = min((int)u, n - 2);
-    const double f = u - (double)m;
-    return T[m] + f * (T[m + 1] - T[m]);
-}
-
-// dT/du of the interpolant (the slope of the segment holding u; zero outside
-// the samples), FP64, for the redshift derivatives of the set-up.
-__device__ __forceinline__ double tab_dT64(const double* __restrict__ T, int n, double u) {
-    if (!(u >= 0.0 && u <= (double)(n - 1))) return 0.0;
-    const int m = min((int)u, n - 2);
-    return T[m + 1] - T[m];
+// Double-float (samples as hi + lo), for the once-per-galaxy set-up (zero
+// points, lambda_eff, c_SSP): T at sample coordinate u, which the caller has
+// found inside the samples, and its slope dT/du (the segment holding u).
+__device__ __forceinline__ Df tab_Tdf(const float* __restrict__ Th, const float* __restrict__ Tl, int n, Df u,
+                                      Df& slope) {
+    const int m = min(max((int)floorf(u.h), 0), n - 2);
+    const Df f = two_sum(u.h - (float)m, u.l);
+    const Df t0{__ldg(Th + m), __ldg(Tl + m)}, t1{__ldg(Th + m + 1), __ldg(Tl + m + 1)};
+    slope = df_sub(t1, t0);
+    return df_add(t0, df_mul(f, slope));
 }
 
 // FP32, for the exact-path epilogues.

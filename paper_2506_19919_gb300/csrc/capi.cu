@@ -441,7 +441,10 @@ sps_status sps_create(sps_ctx** out, const sps_tables* t, const sps_config* cfg_
         }
     }
     if (tab64.empty()) tab64.push_back(0.0);
-    std::vector<float> tab32(tab64.begin(), tab64.end());
+    std::vector<float> tab32(tab64.begin(), tab64.end()), tabl(tab64.size());
+    for (size_t i = 0; i < tab64.size(); ++i) tabl[i] = (float)(tab64[i] - (double)tab32[i]);
+    double gl32[64];
+    gauss_legendre(32, gl32, gl32 + 32);
     ctx->band_p0.assign(t->band_p0, t->band_p0 + B);
     ctx->band_p1.assign(t->band_p1, t->band_p1 + B);
 
@@ -497,10 +500,13 @@ sps_status sps_create(sps_ctx** out, const sps_tables* t, const sps_config* cfg_
         (e = upload(ctx->bp0, t->band_p0, sizeof(double) * B)) != cudaSuccess ||
         (e = upload(ctx->bp1, t->band_p1, sizeof(double) * B)) != cudaSuccess ||
         (e = upload(ctx->tabT, tab32.data(), sizeof(float) * tab32.size())) != cudaSuccess ||
-        (e = upload(ctx->tabT64, tab64.data(), sizeof(double) * tab64.size())) != cudaSuccess ||
+        (e = upload(ctx->tabTl, tabl.data(), sizeof(float) * tabl.size())) != cudaSuccess ||
+        (e = upload(ctx->gl32, gl32, sizeof(gl32))) != cudaSuccess ||
         (e = ctx->lam32.reserve(sizeof(float) * L)) != cudaSuccess ||
         (e = ctx->lamc.reserve(sizeof(float4) * L)) != cudaSuccess ||
         (e = ctx->lamq.reserve(sizeof(float2) * L)) != cudaSuccess ||
+        (e = ctx->lamd.reserve(sizeof(float4) * L)) != cudaSuccess ||
+        (e = ctx->lamdq.reserve(sizeof(float2) * L)) != cudaSuccess ||
         (e = ctx->nonfinite.reserve(64)) != cudaSuccess || (e = ctx->queue.reserve(64)) != cudaSuccess ||
         (e = ctx->err.reserve(64)) != cudaSuccess) {
         delete ctx;
@@ -508,7 +514,8 @@ sps_status sps_create(sps_ctx** out, const sps_tables* t, const sps_config* cfg_
                                                 : cuda_fail(e, "table upload");
     }
     if ((e = launch_lambda_consts(ctx->lam64.as<double>(), L, ctx->lamc.as<float4>(),
-                                  ctx->lam32.as<float>(), ctx->lamq.as<float2>(), 0)) != cudaSuccess ||
+                                  ctx->lam32.as<float>(), ctx->lamq.as<float2>(), ctx->lamd.as<float4>(),
+                                  ctx->lamdq.as<float2>(), 0)) != cudaSuccess ||
         (e = cudaDeviceSynchronize()) != cudaSuccess) {
         delete ctx;
         return cuda_fail(e, "lambda constants");
@@ -520,6 +527,17 @@ sps_status sps_create(sps_ctx** out, const sps_tables* t, const sps_config* cfg_
 
 sps_status sps_destroy(sps_ctx* ctx) {
     delete ctx;
+    return SPS_OK;
+}
+
+// The c_SSP table (deriv 0) or its redshift derivative, galaxies in redshift order.
+static sps_status build_cssp(sps_ctx* ctx, float* out, int deriv, cudaStream_t s) {
+    const int64_t G = ctx->n_gal;
+    CK(ctx->zperm.reserve(sizeof(int32_t) * (2 * (size_t)G + (size_t)zsort_buckets())));
+    int32_t* perm = ctx->zperm.as<int32_t>();
+    CK(launch_zsort(ctx->gal(), nullptr, G, perm, perm + G, perm + 2 * G, s));
+    CK(launch_cssp(ctx->c, ctx->grid(), ctx->gal(), perm, ctx->bp0.as<double>(), ctx->bp1.as<double>(), out, s,
+                   deriv));
     return SPS_OK;
 }
 
@@ -552,12 +570,13 @@ sps_status sps_set_galaxies(sps_ctx* ctx, const float* z, int64_t n_gal, int32_t
     ctx->n_gal = n_gal;
     ctx->has_approx = false;
     ctx->has_dcssp = false;
-    CK(launch_prepare_galaxies(c, ctx->grid(), ctx->lam64.as<double>(), ctx->bp0.as<double>(),
-                               ctx->bp1.as<double>(), ctx->age_edges.as<double>(), ctx->gz.as<float>(),
-                               n_gal, ctx->h0, ctx->om, ctx->glnT.as<float>(), ctx->glT10.as<float>(),
+    CK(ctx->prep.reserve(prepare_scratch_bytes(c, n_gal)));
+    CK(launch_prepare_galaxies(c, ctx->grid(), ctx->bp0.as<double>(), ctx->bp1.as<double>(),
+                               ctx->age_edges.as<double>(), ctx->gl32.as<double>(), ctx->gz.as<float>(), n_gal,
+                               ctx->h0, ctx->om, ctx->glnT.as<float>(), ctx->glT10.as<float>(),
                                ctx->gbins.as<float2>(), ctx->gzp.as<double>(), ctx->gsup.as<int2>(),
                                ctx->ggauss.as<float2>(), ctx->gdust.as<float4>(), ctx->gdtdz.as<float>(),
-                               ctx->gdzp.as<float>(), ctx->gddust.as<float4>(), s));
+                               ctx->gdzp.as<float>(), ctx->gddust.as<float4>(), ctx->prep.p, s));
     if (build_approx) {
         cudaError_t e = ctx->gcssp.reserve(G * B * c.K * sizeof(float));
         if (e != cudaSuccess) {
@@ -565,8 +584,7 @@ sps_status sps_set_galaxies(sps_ctx* ctx, const float* z, int64_t n_gal, int32_t
             return fail(SPS_E_NOMEM, "c_SSP table does not fit in device memory");
         }
         ctx->has_approx = true;
-        CK(launch_cssp(c, ctx->grid(), ctx->gal(), ctx->bp0.as<double>(), ctx->bp1.as<double>(),
-                       ctx->gcssp.as<float>(), s));
+        if (sps_status r = build_cssp(ctx, ctx->gcssp.as<float>(), 0, s); r != SPS_OK) return r;
     }
     CK(cudaStreamSynchronize(s));
     return SPS_OK;
@@ -797,8 +815,7 @@ sps_status sps_loglike_grad_z(sps_ctx* ctx, const float* theta, const int32_t* g
             cudaGetLastError();
             return fail(SPS_E_NOMEM, "the d c_SSP / dz table does not fit in device memory");
         }
-        CK(launch_cssp(c, ctx->grid(), ctx->gal(), ctx->bp0.as<double>(), ctx->bp1.as<double>(),
-                       ctx->gdcssp.as<float>(), s, 1));
+        if (sps_status r = build_cssp(ctx, ctx->gdcssp.as<float>(), 1, s); r != SPS_OK) return r;
         ctx->has_dcssp = true;
     }
     const size_t GB = (size_t)ctx->n_gal * c.n_band;

@@ -69,14 +69,15 @@ struct sps_ctx {
     double gl_x[sps::kMaxGL], gl_w[sps::kMaxGL];
     std::vector<double> band_p0, band_p1;
     // tables
-    DevBuf lam64, lam32, lamc, lamq, ssp, ssp_t, ssp_bf, ssp_t_bf, row_scale, col_scale, age_edges, bp0, bp1;
+    DevBuf lam64, lam32, lamc, lamq, lamd, lamdq, gl32, ssp, ssp_t, ssp_bf, ssp_t_bf, row_scale, col_scale, age_edges, bp0, bp1;
     DevBuf ssp_hi, ssp_lo, ssp_t_hi, ssp_t_lo;   // 3xTF32 halves of the FP32 tables
-    DevBuf tabT, tabT64;                         // tabulated transmission samples
+    DevBuf tabT, tabTl;                          // tabulated transmission samples, high and low parts
     // galaxies
     int64_t n_gal = 0;
     bool has_approx = false;
     DevBuf gz, glnT, glT10, gbins, gzp, gsup, ggauss, gcssp, gdust;
     DevBuf gdtdz, gdzp, gddust;       // redshift derivatives of the per-galaxy set-up
+    DevBuf prep;                      // scratch of the per-galaxy set-up
     DevBuf gdcssp;                    // d c_SSP / dz, built on the first request
     bool has_dcssp = false;
     DevBuf cJz, rowz;                 // exact path: the z accumulators and explicit z term
@@ -104,6 +105,8 @@ struct sps_ctx {
         g.lamc = lamc.as<float4>();
         g.lamq = lamq.as<float2>();
         g.lam64 = lam64.as<double>();
+        g.lamd = lamd.as<float4>();
+        g.lamdq = lamdq.as<float2>();
         g.ssp = ssp.as<float>();
         g.ssp_t = ssp_t.as<float>();
         g.ssp_bf = ssp_bf.as<uint16_t>();
@@ -111,7 +114,7 @@ struct sps_ctx {
         g.row_scale = row_scale.as<float>();
         g.col_scale = col_scale.as<float>();
         g.band_T = tabT.as<float>();
-        g.band_T64 = tabT64.as<double>();
+        g.band_Tl = tabTl.as<float>();
         return g;
     }
     Galaxies gal() const {
@@ -138,11 +141,11 @@ struct sps_ctx {
         if (fork) cudaEventDestroy(fork);
         if (join) cudaEventDestroy(join);
         if (side) cudaStreamDestroy(side);
-        DevBuf* all[] = {&lam64, &lam32, &lamc, &lamq, &ssp, &ssp_t, &ssp_bf, &ssp_t_bf, &row_scale, &col_scale,
+        DevBuf* all[] = {&lam64, &lam32, &lamc, &lamq, &lamd, &lamdq, &gl32, &prep, &ssp, &ssp_t, &ssp_bf, &ssp_t_bf, &row_scale, &col_scale,
                          &age_edges, &bp0, &bp1, &gz, &glnT, &glT10, &gbins, &gzp, &gsup, &ggauss,
                          &gcssp, &gdust, &gdtdz, &gdzp, &gddust, &gdcssp, &cJz, &rowz, &nonfinite, &queue, &err, &W, &V, &Wbar, &cJ, &gbar,
                          &rowinfo, &tcerr, &plainT, &plainC, &hmcm, &pst, &pth, &pll, &pgr,
-                         &pgi, &hmcn, &zperm, &ssp_hi, &ssp_lo, &ssp_t_hi, &ssp_t_lo, &Wlo, &Vlo, &keep, &tabT, &tabT64};
+                         &pgi, &hmcn, &zperm, &ssp_hi, &ssp_lo, &ssp_t_hi, &ssp_t_lo, &Wlo, &Vlo, &keep, &tabT, &tabTl};
         for (DevBuf* b : all) b->release();
         for (auto& b : stage) b.release();
     }

@@ -64,6 +64,8 @@ struct Grid {
     const float4* lamc;      // [L] (q_n / lambda_n, k0, ln(lambda/lambda_V), Drude shape)
     const float2* lamq;      // [L] (lambda, q_n / lambda_n) in FP32
     const double* lam64;     // [L] Angstrom, FP64
+    const float4* lamd;      // [L] lambda and q_n / lambda_n as double-float pairs (hi, lo, hi, lo)
+    const float2* lamdq;     // [L] q_n as a double-float pair
     const float* ssp_t;      // [lam_pad][k_pad] SSP table transposed, FP32 (zero padded)
     const float* ssp;        // [k_pad][lam_pad] SSP table, FP32 (zero padded)
     const uint16_t* ssp_bf;  // [k_pad][lam_pad] SSP table, BF16 bits, row-scaled by 2^-e_i
@@ -71,7 +73,7 @@ struct Grid {
     const float* row_scale;  // [A] 2^e_i
     const float* col_scale;  // [k_pad] 2^e_i of column k = i Zn + j, 0 past K
     const float* band_T;     // tabulated transmission samples, all TABLE bands (FP32)
-    const double* band_T64;  // the same in FP64 (per-galaxy set-up kernels)
+    const float* band_Tl;    // their low parts, sample = T + Tl (per-galaxy set-up kernels)
 };
 
 // Metric-adaptation state of one HMC chain, kept in global memory (read at
@@ -113,14 +115,17 @@ void set_last_error(const char* msg);
 int pointer_location(const void* p, int device);
 
 // Launchers (defined in the .cu files); all return cudaError_t of the launch.
-cudaError_t launch_prepare_galaxies(const Consts& c, const Grid& grid, const double* lam64,
-                                    const double* band_p0, const double* band_p1,
-                                    const double* age_edges_yr, const float* z, int64_t n_gal,
-                                    double h0, double om, float* lnT, float* lT10, float2* bins,
-                                    double* zp, int2* support, float2* gauss, float4* dust_eff,
-                                    float* dtdz, float* dzp, float4* ddust, cudaStream_t s);
-// c_SSP (deriv = 0) or its redshift derivative d c_SSP / dz (deriv = 1)
-cudaError_t launch_cssp(const Consts& c, const Grid& grid, const Galaxies& g,
+// scratch: prepare_scratch_bytes(c, n_gal); gl32: nodes and weights of the 32-node
+// Gauss-Legendre rule on [-1, 1]
+size_t prepare_scratch_bytes(const Consts& c, int64_t n_gal);
+cudaError_t launch_prepare_galaxies(const Consts& c, const Grid& grid, const double* band_p0,
+                                    const double* band_p1, const double* age_edges_yr, const double* gl32,
+                                    const float* z, int64_t n_gal, double h0, double om, float* lnT, float* lT10,
+                                    float2* bins, double* zp, int2* support, float2* gauss, float4* dust_eff,
+                                    float* dtdz, float* dzp, float4* ddust, void* scratch, cudaStream_t s);
+// c_SSP (deriv = 0) or its redshift derivative d c_SSP / dz (deriv = 1); perm: the
+// galaxies in redshift order
+cudaError_t launch_cssp(const Consts& c, const Grid& grid, const Galaxies& g, const int32_t* perm,
                         const double* band_p0, const double* band_p1, float* cssp, cudaStream_t s,
                         int deriv = 0);
 
@@ -149,8 +154,8 @@ cudaError_t launch_exact_fwd(const Consts& c, const Grid& grid, const Galaxies& 
                              const float* theta, const int32_t* gal_idx, int64_t n, int bf16,
                              const float* W32, const uint16_t* Wbf, float* cJ, cudaStream_t s,
                              float* cJz = nullptr);   // with cJz: [r][b][2] sum_n wb' S (1, E)
-cudaError_t launch_lambda_consts(const double* lam, int L, float4* out, float* lam32, float2* lamq,
-                                 cudaStream_t s);
+cudaError_t launch_lambda_consts(const double* lam, int L, float4* out, float* lam32, float2* lamq, float4* lamd,
+                                 float2* lamdq, cudaStream_t s);
 cudaError_t launch_exact_like(const Consts& c, const Galaxies& g, const float* theta,
                               const int32_t* gal_idx, int64_t n, const float* cJ, float* rowinfo,
                               const float* mag_obs, const float* sigma, const uint32_t* mask,
