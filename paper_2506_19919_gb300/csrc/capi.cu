@@ -604,24 +604,29 @@ static sps_status run_exact(sps_ctx* ctx, const float* theta, const int32_t* gid
     const bool tc = tf || (bf16 && ctx->use_tc);
     const int64_t chunk = tc ? (tf ? 65536 : 131072) : 32768;
     const int64_t rows = std::min<int64_t>(n, chunk);
+    const int fsplit = tc ? 1 : simt_fwd_split(c, rows, 64);      // slices of the band sums and of Wbar
+    const int asplit = tc ? 1 : simt_adj_split(c, rows);
     CK(ctx->W.reserve((size_t)rows * c.k_pad * 4));
     if (tf) CK(ctx->Wlo.reserve((size_t)rows * c.k_pad * 4));
-    CK(ctx->cJ.reserve((size_t)rows * c.n_band * 4 * 4));
+    CK(ctx->cJ.reserve((size_t)fsplit * rows * c.n_band * 4 * 4));
     CK(ctx->rowinfo.reserve((size_t)rows * 4 * 4));
     CK(ctx->gbar.reserve((size_t)rows * c.n_band * 4));
-    if (tc) CK(ctx->zperm.reserve(sizeof(int32_t) * (2 * (size_t)rows + (size_t)zsort_buckets())));
-    int32_t* perm = tc ? ctx->zperm.as<int32_t>() : nullptr;
-    int32_t* pos_of = tc ? perm + rows : nullptr;
-    int32_t* zcounts = tc ? perm + 2 * rows : nullptr;
+    // redshift order of the rows, bucket counts, row-tile hulls
+    const int64_t hulls = 2 * ((rows + 127) / 128);
+    CK(ctx->zperm.reserve(sizeof(int32_t) * (2 * (size_t)rows + 2 + (size_t)(zsort_buckets() + hulls))));
+    int32_t* perm = ctx->zperm.as<int32_t>();
+    int32_t* pos_of = perm + rows;
+    int32_t* zcounts = perm + 2 * ((rows + 1) / 2 * 2);
+    uint32_t* hull = reinterpret_cast<uint32_t*>(zcounts + zsort_buckets());
     if (grad_out) {
         CK(ctx->V.reserve((size_t)rows * c.lam_pad * 4));
-        CK(ctx->Wbar.reserve((size_t)rows * c.k_pad * 4));
+        CK(ctx->Wbar.reserve((size_t)asplit * rows * c.k_pad * 4));
         if (tf) CK(ctx->Vlo.reserve((size_t)rows * c.lam_pad * 4));
         CK(ctx->keep.reserve((size_t)rows * (size_t)keep_stride(c) * 4));
     }
     float* keep = grad_out ? ctx->keep.as<float>() : nullptr;
     if (want_z) {
-        CK(ctx->cJz.reserve((size_t)rows * c.n_band * 2 * 4));
+        CK(ctx->cJz.reserve((size_t)fsplit * rows * c.n_band * 2 * 4));
         CK(ctx->rowz.reserve((size_t)rows * 4));
     }
     float* cJz = want_z ? ctx->cJz.as<float>() : nullptr;
@@ -652,9 +657,9 @@ static sps_status run_exact(sps_ctx* ctx, const float* theta, const int32_t* gid
             if (gv.dcssp) gv.dcssp += r0 * c.n_band * c.K;
             gv.n = m;
         }
-        if (tc) CK(launch_zsort(gv, gi, m, perm, pos_of, zcounts, s));
+        CK(launch_zsort(gv, gi, m, perm, pos_of, zcounts, s, hulls));
         CK(launch_exact_weights(c, grid, gv, th, gi, m, bf16, ctx->W.as<float>(), ctx->W.as<uint16_t>(), s,
-                                pos_of, tf ? ctx->Wlo.as<float>() : nullptr, keep));
+                                pos_of, tf ? ctx->Wlo.as<float>() : nullptr, keep, hull));
         if (tc) {
             TcMaps tm;
             const bool ok = tf ? (make_tmap_f32(&tm.a[0], ctx->W.p, c.k_pad, m, c.k_pad, 128) &&
@@ -665,23 +670,23 @@ static sps_status run_exact(sps_ctx* ctx, const float* theta, const int32_t* gid
                                   make_tmap_bf16(&tm.b[0], ctx->ssp_t_bf.p, c.k_pad, c.n_lam, c.k_pad, 256));
             if (!ok) return fail(SPS_E_CUDA, "tensor map encoding failed");
             if (!tf) tm.a[1] = tm.a[0], tm.b[1] = tm.b[0];
-            CK(launch_fwd_tc(tm, tf, c, grid, gv, th, gi, perm, m, ctx->cJ.as<float>(), terr, s, cJz));
+            CK(launch_fwd_tc(tm, tf, c, grid, gv, th, gi, perm, hull, m, ctx->cJ.as<float>(), terr, s, cJz));
         } else {
-            CK(launch_exact_fwd(c, grid, gv, th, gi, m, bf16, ctx->W.as<float>(), ctx->W.as<uint16_t>(),
-                                ctx->cJ.as<float>(), s, cJz));
+            CK(launch_exact_fwd(c, grid, gv, th, gi, perm, m, bf16, ctx->W.as<float>(), ctx->W.as<uint16_t>(),
+                                ctx->cJ.as<float>(), fsplit, s, cJz));
         }
         CK(launch_exact_like(c, gv, th, gi, m, ctx->cJ.as<float>(), ctx->rowinfo.as<float>(), mo, sg,
                              mk, mag_out ? mag_out + r0 * c.n_band : nullptr,
                              ll_out ? ll_out + r0 : nullptr, ctx->gbar.as<float>(), nf, s, cJz, rowz,
-                             ll64_out ? ll64_out + r0 : nullptr));
+                             ll64_out ? ll64_out + r0 : nullptr, fsplit));
         if (grad_out) {
             if (tc) {
                 if (tf)
                     CK(launch_exact_vgen(c, grid, gv, th, gi, m, ctx->gbar.as<float>(), ctx->V.as<float>(),
-                                         nullptr, s, ctx->Vlo.as<float>()));
+                                         nullptr, s, ctx->Vlo.as<float>(), perm, hull));
                 else
                     CK(launch_exact_vgen(c, grid, gv, th, gi, m, ctx->gbar.as<float>(), nullptr,
-                                         ctx->V.as<uint16_t>(), s));
+                                         ctx->V.as<uint16_t>(), s, nullptr, perm, hull));
                 TcMaps tm;
                 const bool ok = tf ? (make_tmap_f32(&tm.a[0], ctx->V.p, c.lam_pad, m, c.lam_pad, 128) &&
                                       make_tmap_f32(&tm.a[1], ctx->Vlo.p, c.lam_pad, m, c.lam_pad, 128) &&
@@ -691,14 +696,14 @@ static sps_status run_exact(sps_ctx* ctx, const float* theta, const int32_t* gid
                                       make_tmap_bf16(&tm.b[0], ctx->ssp_bf.p, c.lam_pad, c.K, c.lam_pad, 224));
                 if (!ok) return fail(SPS_E_CUDA, "tensor map encoding failed");
                 if (!tf) tm.a[1] = tm.a[0], tm.b[1] = tm.b[0];
-                CK(launch_adj_tc(tm, tf, c, grid, m, ctx->Wbar.as<float>(), terr, s));
+                CK(launch_adj_tc(tm, tf, c, grid, m, hull, ctx->Wbar.as<float>(), terr, s));
             } else {
                 CK(launch_exact_vgen(c, grid, gv, th, gi, m, ctx->gbar.as<float>(), ctx->V.as<float>(),
-                                     nullptr, s));
-                CK(launch_exact_adj(c, grid, m, bf16, ctx->V.as<float>(), ctx->Wbar.as<float>(), s));
+                                     nullptr, s, nullptr, perm, hull));
+                CK(launch_exact_adj(c, grid, m, bf16, ctx->V.as<float>(), hull, ctx->Wbar.as<float>(), asplit, s));
             }
             CK(launch_exact_grad(c, gv, th, gi, m, ctx->rowinfo.as<float>(), ctx->Wbar.as<float>(),
-                                 grad_out + r0 * NG, s, rowz, keep));
+                                 grad_out + r0 * NG, s, rowz, keep, pos_of, asplit));
         }
     }
     return SPS_OK;

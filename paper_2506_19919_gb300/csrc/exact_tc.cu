@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(64) k_wait_probe(int ready, uint32_t limit, in
 template <bool TF>
 __global__ void __launch_bounds__(kThreadsTC, 1)
 k_adj_tc(const __grid_constant__ TcMaps tm, const __grid_constant__ Consts c, const Grid grid, int64_t n,
-         float* __restrict__ Wbar, int* err, int tpc) {
+         const uint32_t* __restrict__ hull, float* __restrict__ Wbar, int* err, int tpc) {
     extern __shared__ unsigned char smem_raw[];
     constexpr int ST = TF ? 2 : kAdjStages;
     using R = Ring<kAdjBN, ST, TF>;
@@ -63,22 +63,24 @@ k_adj_tc(const __grid_constant__ TcMaps tm, const __grid_constant__ Consts c, co
     const int m0 = (int)(blockIdx.x / groups) * kTM;
     const int nt0 = (int)(blockIdx.x % groups) * tpc;
     const int n_tiles = min(tpc, n_tiles_all - nt0);
-    const int n_kb = (c.lam_pad + R::kBK - 1) / R::kBK;   // the last block reads zero fill
-    const int kchunk = n_kb;                                // one accumulation per tile
-    const int n_kc = (n_kb + kchunk - 1) / kchunk;
+    // v is zero outside the hull of the rows' supports: the reduction covers its
+    // k-blocks only (the grid's last one reads zero fill); 100,000 rows, six bands:
+    // 0.64 ms against 1.11 ms over the whole grid
+    const int2 hr = row_hull(c, hull, m0);
+    const int kb0 = hr.x / R::kBK, kb1 = (hr.y + R::kBK - 1) / R::kBK;
     tc_setup<ST>(ctl, warp);
     if (warp == 0) {
-        if (lane == 0) tc_produce<kAdjBN, ST, TF>(ctl, ring, tm.a, tm.b, m0, n_tiles, n_kb, err, kchunk, nt0);
+        if (lane == 0) tc_produce<kAdjBN, ST, TF>(ctl, ring, tm.a, tm.b, m0, n_tiles, nt0 * kAdjBN, kb0, kb1,
+                                                          err);
     } else if (warp == 1) {
-        if (lane == 0) tc_mma<kAdjBN, ST, TF>(ctl, ring, n_tiles, n_kb, err, kchunk);
+        if (lane == 0) tc_mma<kAdjBN, ST, TF>(ctl, ring, n_tiles, kb1 - kb0, err);
     } else {
         const int q = warp & 3;
         const int64_t row = (int64_t)m0 + 32 * q + lane;
         const bool live = row < n;
-        for (int item = 0; item < n_tiles * n_kc; ++item) {
-            const int buf = item & 1;
-            const uint32_t use = (uint32_t)(item >> 1);
-            const int nt = item / n_kc, kc = item - nt * n_kc;
+        for (int nt = 0; nt < n_tiles; ++nt) {
+            const int buf = nt & 1;
+            const uint32_t use = (uint32_t)(nt >> 1);
             if (!warp_wait(&ctl->tfull[buf], use & 1u, ctl, err)) break;
             tc::tc_fence_after();
             for (int cc = 0; cc < kAdjBN / 32; ++cc) {
@@ -101,20 +103,11 @@ k_adj_tc(const __grid_constant__ TcMaps tm, const __grid_constant__ Consts c, co
 #pragma unroll
                         for (int t = 0; t < 4; ++t) v[t] = TF ? S[j + t] : S[j + t] * cs[t];
                         if (k + 3 < c.K) {
-                            float4* o = reinterpret_cast<float4*>(orow + k);
-                            if (kc == 0) {
-                                *o = make_float4(v[0], v[1], v[2], v[3]);
-                            } else {
-                                float4 p = *o;
-                                *o = make_float4(p.x + v[0], p.y + v[1], p.z + v[2], p.w + v[3]);
-                            }
+                            *reinterpret_cast<float4*>(orow + k) = make_float4(v[0], v[1], v[2], v[3]);
                         } else {
 #pragma unroll
                             for (int t = 0; t < 4; ++t)
-                                if (k + t < c.K) {
-                                    if (kc == 0) orow[k + t] = v[t];
-                                    else orow[k + t] += v[t];
-                                }
+                                if (k + t < c.K) orow[k + t] = v[t];
                         }
                     }
                 }
@@ -137,14 +130,14 @@ size_t tc_adj_smem(bool tf) {
 }
 
 cudaError_t launch_fwd_tc(const TcMaps& tm, bool tf, const Consts& c, const Grid& grid, const Galaxies& g,
-                          const float* theta, const int32_t* gal_idx, const int32_t* perm, int64_t n, float* cJ,
-                          int* err, cudaStream_t s, float* cJz) {
-    if (cJz) return launch_fwd_tc_z(tm, tf, c, grid, g, theta, gal_idx, perm, n, cJ, err, s, cJz);
-    return fwd_tc_launch<false>(tm, tf, c, grid, g, theta, gal_idx, perm, n, cJ, err, s, nullptr);
+                          const float* theta, const int32_t* gal_idx, const int32_t* perm, const uint32_t* hull,
+                          int64_t n, float* cJ, int* err, cudaStream_t s, float* cJz) {
+    if (cJz) return launch_fwd_tc_z(tm, tf, c, grid, g, theta, gal_idx, perm, hull, n, cJ, err, s, cJz);
+    return fwd_tc_launch<false>(tm, tf, c, grid, g, theta, gal_idx, perm, hull, n, cJ, err, s, nullptr);
 }
 
-cudaError_t launch_adj_tc(const TcMaps& tm, bool tf, const Consts& c, const Grid& grid, int64_t n, float* Wbar,
-                          int* err, cudaStream_t s) {
+cudaError_t launch_adj_tc(const TcMaps& tm, bool tf, const Consts& c, const Grid& grid, int64_t n,
+                          const uint32_t* hull, float* Wbar, int* err, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     // n tiles per block (SPS_ADJ_TPC overrides; tuning only): 3 keeps the
     // TMEM double buffer busy while the row block's 2 blocks share V in L2
@@ -160,11 +153,11 @@ cudaError_t launch_adj_tc(const TcMaps& tm, bool tf, const Consts& c, const Grid
     if (tf) {
         e = cudaFuncSetAttribute(k_adj_tc<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        k_adj_tc<true><<<blocks, kThreadsTC, smem, s>>>(tm, c, grid, n, Wbar, err, tpc);
+        k_adj_tc<true><<<blocks, kThreadsTC, smem, s>>>(tm, c, grid, n, hull, Wbar, err, tpc);
     } else {
         e = cudaFuncSetAttribute(k_adj_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        k_adj_tc<false><<<blocks, kThreadsTC, smem, s>>>(tm, c, grid, n, Wbar, err, tpc);
+        k_adj_tc<false><<<blocks, kThreadsTC, smem, s>>>(tm, c, grid, n, hull, Wbar, err, tpc);
     }
     return cudaGetLastError();
 }

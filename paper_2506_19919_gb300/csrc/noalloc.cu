@@ -25,6 +25,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstring>
 #include <mutex>
 #include <string>
@@ -139,6 +140,9 @@ extern "C" sps_status sps_photometry_exact_noalloc(sps_ctx* ctx, const float* th
         }
         base = a.ptr;
     }
+    // wavelength parts of the contraction as far as the scratch holds their slices
+    const size_t a_slice = (size_t)n * c.n_band * 4 * sizeof(float);
+    const int nsplit = sps::simt_fwd_split(c, n, (int)std::min<size_t>((kScratchBytes - w_bytes) / a_slice, 64));
     float* W = static_cast<float*>(base);
     float* A = reinterpret_cast<float*>(static_cast<unsigned char*>(base) + w_bytes);
     cudaStream_t s = (cudaStream_t)stream;
@@ -149,10 +153,11 @@ extern "C" sps_status sps_photometry_exact_noalloc(sps_ctx* ctx, const float* th
     if ((e = cudaMemsetAsync(nf, 0, sizeof(int), s)) != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
     if ((e = sps::launch_exact_weights(c, grid, gal, theta, gal_idx, n, 0, W, nullptr, s)) != cudaSuccess)
         return cuda_fail(e, "weights launch");
-    if ((e = sps::launch_exact_fwd(c, grid, gal, theta, gal_idx, n, 0, W, nullptr, A, s)) != cudaSuccess)
+    if ((e = sps::launch_exact_fwd(c, grid, gal, theta, gal_idx, nullptr, n, 0, W, nullptr, A, nsplit, s)) != cudaSuccess)
         return cuda_fail(e, "contraction launch");
     if ((e = sps::launch_exact_like(c, gal, theta, gal_idx, n, A, nullptr, nullptr, nullptr, nullptr,
-                                    mag_out, nullptr, nullptr, nf, s)) != cudaSuccess)
+                                    mag_out, nullptr, nullptr, nf, s, nullptr, nullptr, nullptr,
+                                    nsplit)) != cudaSuccess)
         return cuda_fail(e, "magnitude launch");
     int flag = 0;
     if ((e = cudaMemcpyAsync(&flag, nf, sizeof(int), cudaMemcpyDeviceToHost, s)) != cudaSuccess)

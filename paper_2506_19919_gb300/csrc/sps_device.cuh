@@ -52,6 +52,21 @@ __device__ __forceinline__ double warp_sum_d(double v) {
 }
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
 
+// ---------------------------------------------------------------- row tiles
+// Rows ordered by redshift are contracted in tiles that look at one wavelength
+// range, the hull of their band supports.  k_weights collects it per kHullRows
+// positions as (max of n_lam - lo, max of hi), from zeroed memory; row_hull
+// gives the range of the tile holding position pos, widened to multiples of 64
+// inside the padded grid (never empty; the whole grid without a hull).
+constexpr int kHullRows = 128;
+__device__ __forceinline__ int2 row_hull(const Consts& c, const uint32_t* __restrict__ hull, int64_t pos) {
+    if (!hull) return make_int2(0, c.lam_pad);
+    const uint2 h = reinterpret_cast<const uint2*>(hull)[pos / kHullRows];
+    const int lo = c.n_lam - (int)h.x, hi = (int)h.y;
+    if (hi <= lo) return make_int2(0, min(64, c.lam_pad));
+    return make_int2(lo & ~63, min((hi + 63) & ~63, c.lam_pad));
+}
+
 // ---------------------------------------------------------------- triweight
 // CDF of Eq. triweight: with u = x/3 clipped to [-1, 1],
 // 1/2 + (35/32)(u - u^3 + 3u^5/5 - u^7/7).

@@ -148,11 +148,18 @@ cudaError_t launch_exact_weights(const Consts& c, const Grid& grid, const Galaxi
                                  int bf16, float* W32, uint16_t* Wbf, cudaStream_t s,
                                  const int32_t* pos_of = nullptr,    // W row of each row (or itself)
                                  float* W32lo = nullptr,             // with W32lo: W32 = TF32 hi, W32lo = lo
-                                 float* keep = nullptr);             // with keep: the row's weight arrays
+                                 float* keep = nullptr,              // with keep: the row's weight arrays
                                                                      // (keep_stride floats per row)
-cudaError_t launch_exact_fwd(const Consts& c, const Grid& grid, const Galaxies& g,
-                             const float* theta, const int32_t* gal_idx, int64_t n, int bf16,
-                             const float* W32, const uint16_t* Wbf, float* cJ, cudaStream_t s,
+                                 uint32_t* hull = nullptr);          // with hull (zeroed): the row tiles' hulls
+// SIMT contractions (exact_simt.cu).  The forward writes nsplit slices of cJ
+// ([n][B][4] each; cJz [n][B][2]), the adjoint nsplit slices of Wbar ([n][k_pad]),
+// which the likelihood and gradient kernels add up in order; simt_*_split
+// chooses the counts.  perm: the row at each position of W and V.
+int simt_fwd_split(const Consts& c, int64_t n, int max_split);
+int simt_adj_split(const Consts& c, int64_t n);
+cudaError_t launch_exact_fwd(const Consts& c, const Grid& grid, const Galaxies& g, const float* theta,
+                             const int32_t* gal_idx, const int32_t* perm, int64_t n, int bf16, const float* W32,
+                             const uint16_t* Wbf, float* cJ, int nsplit, cudaStream_t s,
                              float* cJz = nullptr);   // with cJz: [r][b][2] sum_n wb' S (1, E)
 cudaError_t launch_lambda_consts(const double* lam, int L, float4* out, float* lam32, float2* lamq, float4* lamd,
                                  float2* lamdq, cudaStream_t s);
@@ -163,18 +170,23 @@ cudaError_t launch_exact_like(const Consts& c, const Galaxies& g, const float* t
                               cudaStream_t s,
                               const float* cJz = nullptr,   // with cJz: rowz[r] = the explicit
                               float* rowz = nullptr,        // (fixed-weights) part of dlogL/dz
-                              double* ll64_out = nullptr);  // log L in FP64 (the samplers' accept)
+                              double* ll64_out = nullptr,   // log L in FP64 (the samplers' accept)
+                              int nsplit = 1);              // slices of cJ and cJz
 cudaError_t launch_exact_vgen(const Consts& c, const Grid& grid, const Galaxies& g,
                               const float* theta, const int32_t* gal_idx, int64_t n,
                               const float* gbar, float* V32, uint16_t* Vbf, cudaStream_t s,
-                              float* V32lo = nullptr);   // with V32lo: V32 = TF32 hi, V32lo = lo
-cudaError_t launch_exact_adj(const Consts& c, const Grid& grid, int64_t n, int bf16,
-                             const float* V32, float* Wbar, cudaStream_t s);
+                              float* V32lo = nullptr,    // with V32lo: V32 = TF32 hi, V32lo = lo
+                              const int32_t* perm = nullptr,      // the row at each position of V
+                              const uint32_t* hull = nullptr);    // v inside the row tiles' hulls only
+cudaError_t launch_exact_adj(const Consts& c, const Grid& grid, int64_t n, int bf16, const float* V32,
+                             const uint32_t* hull, float* Wbar, int nsplit, cudaStream_t s);
 cudaError_t launch_exact_grad(const Consts& c, const Galaxies& g, const float* theta,
                               const int32_t* gal_idx, int64_t n, const float* rowinfo,
                               const float* Wbar, float* grad_out, cudaStream_t s,
                               const float* rowz = nullptr,    // with rowz: 13 columns, z last
-                              const float* keep = nullptr);   // weight arrays kept by the weights kernel
+                              const float* keep = nullptr,    // weight arrays kept by the weights kernel
+                              const int32_t* pos_of = nullptr,   // the position of each row in Wbar
+                              int nsplit = 1);                   // slices of Wbar
 // Floats per row of the kept weight arrays: M (FP64, two floats), then
 // m, dm/dtau, dm/dalpha, dm/dbeta, pi, w over the age bins and q over the
 // metallicity bins; a multiple of 4 floats, so that every row's M is 8-byte
@@ -190,18 +202,19 @@ struct TcMaps {
 size_t tc_fwd_smem(bool tf);
 size_t tc_adj_smem(bool tf);
 cudaError_t launch_fwd_tc(const TcMaps& tm, bool tf, const Consts& c, const Grid& grid, const Galaxies& g,
-                          const float* theta, const int32_t* gal_idx, const int32_t* perm, int64_t n, float* cJ,
-                          int* err, cudaStream_t s, float* cJz = nullptr);
+                          const float* theta, const int32_t* gal_idx, const int32_t* perm, const uint32_t* hull,
+                          int64_t n, float* cJ, int* err, cudaStream_t s, float* cJz = nullptr);
 cudaError_t launch_fwd_tc_z(const TcMaps& tm, bool tf, const Consts& c, const Grid& grid, const Galaxies& g,
-                            const float* theta, const int32_t* gal_idx, const int32_t* perm, int64_t n,
-                            float* cJ, int* err, cudaStream_t s, float* cJz);   // exact_tc_z.cu
-cudaError_t launch_adj_tc(const TcMaps& tm, bool tf, const Consts& c, const Grid& grid, int64_t n, float* Wbar,
-                          int* err, cudaStream_t s);
+                            const float* theta, const int32_t* gal_idx, const int32_t* perm, const uint32_t* hull,
+                            int64_t n, float* cJ, int* err, cudaStream_t s, float* cJz);   // exact_tc_z.cu
+cudaError_t launch_adj_tc(const TcMaps& tm, bool tf, const Consts& c, const Grid& grid, int64_t n,
+                          const uint32_t* hull, float* Wbar, int* err, cudaStream_t s);
 // Rows ordered by redshift (bucketed in log(1+z)): perm[pos] = row,
-// pos_of[row] = pos; counts is scratch of zsort_buckets() ints.
+// pos_of[row] = pos; counts is scratch of zsort_buckets() ints, zeroed with the
+// `extra` ints after it.
 int zsort_buckets();
 cudaError_t launch_zsort(const Galaxies& g, const int32_t* gal_idx, int64_t n, int32_t* perm,
-                         int32_t* pos_of, int32_t* counts, cudaStream_t s);
+                         int32_t* pos_of, int32_t* counts, cudaStream_t s, int64_t extra = 0);
 
 // Plain per-galaxy forward-mode path (comparison baseline).
 size_t plain_scratch_bytes_per_row(const Consts& c);
