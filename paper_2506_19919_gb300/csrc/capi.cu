@@ -604,8 +604,8 @@ static sps_status run_exact(sps_ctx* ctx, const float* theta, const int32_t* gid
     const bool tc = tf || (bf16 && ctx->use_tc);
     const int64_t chunk = tc ? (tf ? 65536 : 131072) : 32768;
     const int64_t rows = std::min<int64_t>(n, chunk);
-    const int fsplit = tc ? 1 : simt_fwd_split(c, rows, 64);      // slices of the band sums and of Wbar
-    const int asplit = tc ? 1 : simt_adj_split(c, rows);
+    const int fsplit = tc ? tc_fwd_split(c, rows, tf) : simt_fwd_split(c, rows, 64);   // slices of the band sums
+    const int asplit = tc ? tc_adj_split(c, rows) : simt_adj_split(c, rows);         // and of Wbar
     CK(ctx->W.reserve((size_t)rows * c.k_pad * 4));
     if (tf) CK(ctx->Wlo.reserve((size_t)rows * c.k_pad * 4));
     CK(ctx->cJ.reserve((size_t)fsplit * rows * c.n_band * 4 * 4));
@@ -670,7 +670,7 @@ static sps_status run_exact(sps_ctx* ctx, const float* theta, const int32_t* gid
                                   make_tmap_bf16(&tm.b[0], ctx->ssp_t_bf.p, c.k_pad, c.n_lam, c.k_pad, 256));
             if (!ok) return fail(SPS_E_CUDA, "tensor map encoding failed");
             if (!tf) tm.a[1] = tm.a[0], tm.b[1] = tm.b[0];
-            CK(launch_fwd_tc(tm, tf, c, grid, gv, th, gi, perm, hull, m, ctx->cJ.as<float>(), terr, s, cJz));
+            CK(launch_fwd_tc(tm, tf, c, grid, gv, th, gi, perm, hull, m, ctx->cJ.as<float>(), fsplit, terr, s, cJz));
         } else {
             CK(launch_exact_fwd(c, grid, gv, th, gi, perm, m, bf16, ctx->W.as<float>(), ctx->W.as<uint16_t>(),
                                 ctx->cJ.as<float>(), fsplit, s, cJz));
@@ -696,7 +696,7 @@ static sps_status run_exact(sps_ctx* ctx, const float* theta, const int32_t* gid
                                       make_tmap_bf16(&tm.b[0], ctx->ssp_bf.p, c.lam_pad, c.K, c.lam_pad, 224));
                 if (!ok) return fail(SPS_E_CUDA, "tensor map encoding failed");
                 if (!tf) tm.a[1] = tm.a[0], tm.b[1] = tm.b[0];
-                CK(launch_adj_tc(tm, tf, c, grid, m, hull, ctx->Wbar.as<float>(), terr, s));
+                CK(launch_adj_tc(tm, tf, c, grid, m, hull, ctx->Wbar.as<float>(), asplit, terr, s));
             } else {
                 CK(launch_exact_vgen(c, grid, gv, th, gi, m, ctx->gbar.as<float>(), ctx->V.as<float>(),
                                      nullptr, s, nullptr, perm, hull));

@@ -347,7 +347,6 @@ k_adj_simt(const __grid_constant__ Consts c, const Grid grid, int64_t n, const f
 // (shared memory feeds 64 FMAs per 16-byte load instead of 32) but leaves SMs
 // idle when the rows are few: the small tile where 128-row tiles would give
 // under a block per SM even with every split.
-constexpr int kSms = 152;
 bool small_tile(int64_t n, int64_t units_per_row_tile) {
     return (n + 127) / 128 * units_per_row_tile < 2 * kSms;
 }

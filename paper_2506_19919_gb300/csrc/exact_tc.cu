@@ -63,17 +63,23 @@ k_adj_tc(const __grid_constant__ TcMaps tm, const __grid_constant__ Consts c, co
     const int m0 = (int)(blockIdx.x / groups) * kTM;
     const int nt0 = (int)(blockIdx.x % groups) * tpc;
     const int n_tiles = min(tpc, n_tiles_all - nt0);
+
     // v is zero outside the hull of the rows' supports: the reduction covers its
     // k-blocks only (the grid's last one reads zero fill); 100,000 rows, six bands:
     // 0.64 ms against 1.11 ms over the whole grid
     const int2 hr = row_hull(c, hull, m0);
-    const int kb0 = hr.x / R::kBK, kb1 = (hr.y + R::kBK - 1) / R::kBK;
+    // and of these the block takes part blockIdx.y of gridDim.y, into its own
+    // slice of Wbar
+    const int kb_lo = hr.x / R::kBK, n_all = (hr.y + R::kBK - 1) / R::kBK - kb_lo;
+    const int kb0 = kb_lo + n_all * (int)blockIdx.y / (int)gridDim.y;
+    const int kb1 = kb_lo + n_all * ((int)blockIdx.y + 1) / (int)gridDim.y;
+    const bool none = kb0 >= kb1;                          // fewer k-blocks than parts: a slice of zeros
     tc_setup<ST>(ctl, warp);
     if (warp == 0) {
-        if (lane == 0) tc_produce<kAdjBN, ST, TF>(ctl, ring, tm.a, tm.b, m0, n_tiles, nt0 * kAdjBN, kb0, kb1,
-                                                          err);
+        if (lane == 0 && !none)
+            tc_produce<kAdjBN, ST, TF>(ctl, ring, tm.a, tm.b, m0, n_tiles, nt0 * kAdjBN, kb0, kb1, err);
     } else if (warp == 1) {
-        if (lane == 0) tc_mma<kAdjBN, ST, TF>(ctl, ring, n_tiles, kb1 - kb0, err);
+        if (lane == 0) tc_mma<kAdjBN, ST, TF>(ctl, ring, none ? 0 : n_tiles, kb1 - kb0, err);
     } else {
         const int q = warp & 3;
         const int64_t row = (int64_t)m0 + 32 * q + lane;
@@ -81,16 +87,22 @@ k_adj_tc(const __grid_constant__ TcMaps tm, const __grid_constant__ Consts c, co
         for (int nt = 0; nt < n_tiles; ++nt) {
             const int buf = nt & 1;
             const uint32_t use = (uint32_t)(nt >> 1);
-            if (!warp_wait(&ctl->tfull[buf], use & 1u, ctl, err)) break;
-            tc::tc_fence_after();
+            if (!none) {
+                if (!warp_wait(&ctl->tfull[buf], use & 1u, ctl, err)) break;
+                tc::tc_fence_after();
+            }
             for (int cc = 0; cc < kAdjBN / 32; ++cc) {
                 float S[32];
-                tc::tmem_ld32(ctl->tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * kAdjBN + cc * 32), S);
+                if (none) {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) S[j] = 0.0f;
+                } else
+                    tc::tmem_ld32(ctl->tmem_base + ((uint32_t)(32 * q) << 16) + (uint32_t)(buf * kAdjBN + cc * 32), S);
                 const int k0 = (nt0 + nt) * kAdjBN + cc * 32;
                 if (live) {
                     // 16-byte stores (k_pad is a multiple of 64, k0 of 32): a lane
                     // owns one row, so each store covers half a sector, not an eighth
-                    float* orow = Wbar + row * c.k_pad;
+                    float* orow = Wbar + ((int64_t)blockIdx.y * n + row) * c.k_pad;
 #pragma unroll
                     for (int j = 0; j < 32; j += 4) {
                         const int k = k0 + j;
@@ -112,14 +124,45 @@ k_adj_tc(const __grid_constant__ TcMaps tm, const __grid_constant__ Consts c, co
                     }
                 }
             }
-            tc::tc_fence_before();
-            tc::mbar_arrive(&ctl->tempty[buf]);
+            if (!none) {
+                tc::tc_fence_before();
+                tc::mbar_arrive(&ctl->tempty[buf]);
+            }
         }
     }
     tc_teardown<ST>(ctl, warp);
 }
 
+// n tiles per block: 3 keeps the TMEM double buffer busy while the row block's
+// 2 blocks share V in L2 (measured 2-7% faster than one block streaming V for
+// all 6 tiles); 1 while that leaves SMs without a block.
+int adj_tpc(const Consts& c, int64_t n) {
+    const int n_tiles_all = (c.K + kAdjBN - 1) / kAdjBN;
+    if (const char* v = std::getenv("SPS_ADJ_TPC")) return std::max(1, std::min(std::atoi(v), n_tiles_all));
+    const int64_t mt = (n + kTM - 1) / kTM;
+    return mt * ((n_tiles_all + 2) / 3) < kSms ? 1 : std::min(3, n_tiles_all);
+}
+
 }  // namespace
+
+// Parts of the forward's wavelength tiles: one block per SM runs a row tile, so
+// fewer row tiles than SMs leave the rest idle; they get as many parts as fit
+// (100 rows, 107 x 12 x 5994 grid, BF16: log L + gradient 197 us against 573 in
+// one part).  From one row tile per SM on the parts only add set-ups and slices
+// (100,000 rows in 3 parts: 2.04 ms against 1.96).
+int tc_fwd_split(const Consts& c, int64_t n, bool tf) {
+    const int64_t mt = (n + kTM - 1) / kTM;
+    const int bn = tf ? kFwdBNtf : kFwdBN;
+    const int most = std::min(24, (c.n_lam + bn - 1) / bn);
+    return (int)std::max<int64_t>(1, std::min<int64_t>(kSms / mt, most));
+}
+// Parts of the adjoint's reduction: few row tiles only (each part writes a
+// slice of Wbar that the gradient kernel reads back).
+int tc_adj_split(const Consts& c, int64_t n) {
+    const int n_tiles_all = (c.K + kAdjBN - 1) / kAdjBN, tpc = adj_tpc(c, n);
+    const int64_t blocks = (n + kTM - 1) / kTM * ((n_tiles_all + tpc - 1) / tpc);
+    return (int)std::max<int64_t>(1, std::min<int64_t>(kSms / blocks, 8));
+}
 
 size_t tc_fwd_smem(bool tf) {
     return (tf ? Ring<kFwdBNtf, kFwdStagesTf, true>::kBytes : Ring<kFwdBN, kFwdStages, false>::kBytes) + 256 +
@@ -131,23 +174,18 @@ size_t tc_adj_smem(bool tf) {
 
 cudaError_t launch_fwd_tc(const TcMaps& tm, bool tf, const Consts& c, const Grid& grid, const Galaxies& g,
                           const float* theta, const int32_t* gal_idx, const int32_t* perm, const uint32_t* hull,
-                          int64_t n, float* cJ, int* err, cudaStream_t s, float* cJz) {
-    if (cJz) return launch_fwd_tc_z(tm, tf, c, grid, g, theta, gal_idx, perm, hull, n, cJ, err, s, cJz);
-    return fwd_tc_launch<false>(tm, tf, c, grid, g, theta, gal_idx, perm, hull, n, cJ, err, s, nullptr);
+                          int64_t n, float* cJ, int nsplit, int* err, cudaStream_t s, float* cJz) {
+    if (cJz) return launch_fwd_tc_z(tm, tf, c, grid, g, theta, gal_idx, perm, hull, n, cJ, nsplit, err, s, cJz);
+    return fwd_tc_launch<false>(tm, tf, c, grid, g, theta, gal_idx, perm, hull, n, cJ, nsplit, err, s, nullptr);
 }
 
 cudaError_t launch_adj_tc(const TcMaps& tm, bool tf, const Consts& c, const Grid& grid, int64_t n,
-                          const uint32_t* hull, float* Wbar, int* err, cudaStream_t s) {
+                          const uint32_t* hull, float* Wbar, int nsplit, int* err, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    // n tiles per block (SPS_ADJ_TPC overrides; tuning only): 3 keeps the
-    // TMEM double buffer busy while the row block's 2 blocks share V in L2
-    // (measured 2-7% faster than one block streaming V for all 6 tiles)
     const int n_tiles_all = (c.K + kAdjBN - 1) / kAdjBN;
-    int tpc = 3;
-    if (const char* v = std::getenv("SPS_ADJ_TPC")) tpc = std::atoi(v);
-    tpc = std::max(1, std::min(tpc, n_tiles_all));
+    const int tpc = adj_tpc(c, n);
     const int groups = (n_tiles_all + tpc - 1) / tpc;
-    const unsigned blocks = (unsigned)(((n + kTM - 1) / kTM) * groups);
+    const dim3 blocks((unsigned)(((n + kTM - 1) / kTM) * groups), nsplit);
     const size_t smem = tc_adj_smem(tf);
     cudaError_t e;
     if (tf) {

@@ -252,10 +252,13 @@ k_fwd_tc(const __grid_constant__ TcMaps tm, const __grid_constant__ Consts c, co
     // the wavelength tiles cover the hull of the rows' band supports only (bands
     // over 360-970 nm: 44% of the production grid); nothing outside it has weight.
     // 100,000 rows, six bands, BF16: 1.39 ms against 1.89 ms over the whole grid
+    // of these tiles the block takes part blockIdx.y of gridDim.y
     const int2 hr = row_hull(c, hull, m0);
-    const int y0 = hr.x;
     const int lam_end = min(hr.y, c.n_lam);
-    const int n_tiles = (lam_end - y0 + BN - 1) / BN;
+    const int n_all = (lam_end - hr.x + BN - 1) / BN;
+    const int t0 = n_all * (int)blockIdx.y / (int)gridDim.y;
+    const int n_tiles = n_all * ((int)blockIdx.y + 1) / (int)gridDim.y - t0;
+    const int y0 = hr.x + t0 * BN;
     const int n_kb = (c.k_pad + R::kBK - 1) / R::kBK;
     const int epi_threads = (int)blockDim.x - 64;
     tc_setup<ST>(ctl, warp, epi_threads);
@@ -490,19 +493,19 @@ k_fwd_tc(const __grid_constant__ TcMaps tm, const __grid_constant__ Consts c, co
             tc::tc_fence_before();
             tc::mbar_arrive(&ctl->tempty[buf]);
         }
-        // cJ is zeroed before the launch; a (row, band) gets one addend per
-        // column half, so the sum does not depend on their order
+        // the block's slice of cJ is zeroed before the launch; a (row, band) gets
+        // one addend per column half, so the sum does not depend on their order
         if (valid && !ctl->abort) {
 #pragma unroll
             for (int k = 0; k < NB; ++k)
                 if (b0 + k < b_end) {
-                    float* o = cJ + (row * B + b0 + k) * 4;
+                    float* o = cJ + (((int64_t)blockIdx.y * n + row) * B + b0 + k) * 4;
                     atomicAdd(o + 0, acc[k][0]);
                     atomicAdd(o + 1, acc[k][1]);
                     atomicAdd(o + 2, acc[k][2]);
                     atomicAdd(o + 3, acc[k][3]);
                     if (KZ) {
-                        float* oz = cJz + (row * B + b0 + k) * 2;
+                        float* oz = cJz + (((int64_t)blockIdx.y * n + row) * B + b0 + k) * 2;
                         atomicAdd(oz + 0, accz[k][0]);
                         atomicAdd(oz + 1, accz[k][1]);
                     }
@@ -518,18 +521,18 @@ k_fwd_tc(const __grid_constant__ TcMaps tm, const __grid_constant__ Consts c, co
 template <bool KZ>
 cudaError_t fwd_tc_launch(const TcMaps& tm, bool tf, const Consts& c, const Grid& grid, const Galaxies& g,
                           const float* theta, const int32_t* gal_idx, const int32_t* perm, const uint32_t* hull,
-                          int64_t n, float* cJ, int* err, cudaStream_t s, float* cJz) {
+                          int64_t n, float* cJ, int nsplit, int* err, cudaStream_t s, float* cJz) {
     if (n <= 0) return cudaSuccess;
     static_assert(kHullRows % kTM == 0, "a tile lies in one hull");
-    const unsigned blocks = (unsigned)((n + kTM - 1) / kTM);
+    const dim3 blocks((unsigned)((n + kTM - 1) / kTM), nsplit);
     const size_t smem = tc_fwd_smem(tf);
     const int groups = (c.n_band + kFwdGroupBands - 1) / kFwdGroupBands;   // <= 4 (B <= 32)
     const int halves = groups == 1 ? 2 : 1;
     const int threads = 64 + 32 * 4 * groups * halves;
-    cudaError_t e = cudaMemsetAsync(cJ, 0, (size_t)n * c.n_band * 4 * sizeof(float), s);
+    cudaError_t e = cudaMemsetAsync(cJ, 0, (size_t)nsplit * n * c.n_band * 4 * sizeof(float), s);
     if (e != cudaSuccess) return e;
     if (cJz) {
-        e = cudaMemsetAsync(cJz, 0, (size_t)n * c.n_band * 2 * sizeof(float), s);
+        e = cudaMemsetAsync(cJz, 0, (size_t)nsplit * n * c.n_band * 2 * sizeof(float), s);
         if (e != cudaSuccess) return e;
     }
     auto go = [&](auto kern) -> cudaError_t {

@@ -13,6 +13,7 @@ constexpr int kMaxAges = SPS_MAX_AGES;   // bins per row held in shared memory
 constexpr int kMaxMets = SPS_MAX_METS;
 constexpr int kMaxBands = SPS_MAX_BANDS;
 constexpr int kMaxGL = 16;
+constexpr int kSms = 152;                // SMs of a GB300 (tile and split rules)
 constexpr int kMaxPanels = 512;          // SFH panels per row (checked on the host)
 constexpr int kKTileMax = 41;            // ceil(K / 32) held in registers: K <= 1312
 constexpr int kWarpsApprox = 4;          // warps per block of the fused approximate kernel
@@ -203,12 +204,17 @@ size_t tc_fwd_smem(bool tf);
 size_t tc_adj_smem(bool tf);
 cudaError_t launch_fwd_tc(const TcMaps& tm, bool tf, const Consts& c, const Grid& grid, const Galaxies& g,
                           const float* theta, const int32_t* gal_idx, const int32_t* perm, const uint32_t* hull,
-                          int64_t n, float* cJ, int* err, cudaStream_t s, float* cJz = nullptr);
+                          int64_t n, float* cJ, int nsplit, int* err, cudaStream_t s, float* cJz = nullptr);
 cudaError_t launch_fwd_tc_z(const TcMaps& tm, bool tf, const Consts& c, const Grid& grid, const Galaxies& g,
                             const float* theta, const int32_t* gal_idx, const int32_t* perm, const uint32_t* hull,
-                            int64_t n, float* cJ, int* err, cudaStream_t s, float* cJz);   // exact_tc_z.cu
+                            int64_t n, float* cJ, int nsplit, int* err, cudaStream_t s,
+                            float* cJz);   // exact_tc_z.cu
 cudaError_t launch_adj_tc(const TcMaps& tm, bool tf, const Consts& c, const Grid& grid, int64_t n,
-                          const uint32_t* hull, float* Wbar, int* err, cudaStream_t s);
+                          const uint32_t* hull, float* Wbar, int nsplit, int* err, cudaStream_t s);
+// parts of the forward's wavelength tiles and of the adjoint's reduction, each
+// writing its own slice of cJ / Wbar as in the SIMT contractions
+int tc_fwd_split(const Consts& c, int64_t n, bool tf);
+int tc_adj_split(const Consts& c, int64_t n);
 // Rows ordered by redshift (bucketed in log(1+z)): perm[pos] = row,
 // pos_of[row] = pos; counts is scratch of zsort_buckets() ints, zeroed with the
 // `extra` ints after it.
