@@ -256,7 +256,7 @@ k_exact_vgen(const __grid_constant__ Consts c, const Grid grid, const Galaxies g
             float wb = lq.y;
             if (kind == 1) {
                 const float u = (lq.x - gp.x) * gsv;
-                wb *= exp2f(-(u * u));
+                wb *= ex2_(-(u * u));
             } else if (kind == 2) {
                 wb *= tab_T32(grid.band_T + c.tab_off[b], c.tab_n[b], (lq.x - gp.x) * -gp.y);
             }
@@ -284,10 +284,10 @@ k_exact_vgen(const __grid_constant__ Consts c, const Grid grid, const Galaxies g
                 const float4 La = grid.lamc[nn];
                 const float4 Lb = (nn + 1 < c.n_lam) ? grid.lamc[nn + 1] : La;
                 const float2 pa = __fmul2_rn(dl2, make_float2(La.z, Lb.z));
-                const float2 pw = make_float2(exp2f(pa.x), exp2f(pa.y));
+                const float2 pw = make_float2(ex2_(pa.x), ex2_(pa.y));
                 const float2 base = __ffma2_rn(make_float2(La.y, Lb.y), pw, __fmul2_rn(eb2, make_float2(La.w, Lb.w)));
                 const float2 ea = __fmul2_rn(cA2, base);
-                const float2 E = make_float2(exp2f(ea.x), exp2f(ea.y));
+                const float2 E = make_float2(ex2_(ea.x), ex2_(ea.y));
                 const float2 F = __ffma2_rn(omf2, E, ff2);
                 const float2 v = __fmul2_rn(F, sum);
                 out = (uint32_t)f_to_bf16(v.x) | ((uint32_t)f_to_bf16(v.y) << 16);

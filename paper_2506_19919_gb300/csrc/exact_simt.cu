@@ -234,16 +234,16 @@ k_fwd_simt(const __grid_constant__ Consts c, const Grid grid, const Galaxies g, 
                         float wz = 0.0f;
                         if (kind == 1) {
                             const float u = (lamt[nl] - gg.x) * gg.y;
-                            wb *= __expf(-0.5f * u * u);
+                            wb *= expf_(-0.5f * u * u);
                             if (KZ) wz = -wb * lamt[nl] * u * fz;       // q T' with T' = -u T / s
                         } else if (kind == 2) {
                             const float ut = (lamt[nl] - gg.x) * -gg.y;
                             wb *= tab_T32(tabT, tabn, ut);
                             if (KZ) wz = L4.x * lamt[nl] * tab_dT32(tabT, tabn, ut) * fz;
                         }
-                        const float pw = __expf(rd.y * L4.z);
+                        const float pw = expf_(rd.y * L4.z);
                         const float base = L4.y * pw + rd.w * L4.w;
-                        const float E = exp2f(-0.4f * kLog2_10f * rd.x * base);
+                        const float E = ex2_(-0.4f * kLog2_10f * rd.x * base);
                         const float dterm = L4.y * pw * L4.z - (rd.w > 0.0f ? 1.9f * L4.w : 0.0f);
                         const float Sn = (j & 1) ? acc[i][j / 2].y : acc[i][j / 2].x;
                         const float S = Sn * wb;

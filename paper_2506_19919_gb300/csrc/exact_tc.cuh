@@ -403,9 +403,9 @@ k_fwd_tc(const __grid_constant__ TcMaps tm, const __grid_constant__ Consts c, co
                         for (int jj = 0; jj < CG; ++jj) {
                             const float4 L4 = cst4[h * CG + jj];
                             lm[jj] = cstl[h * CG + jj];
-                            const float ypw = L4.y * exp2f(dl2 * L4.z);      // k0 (l / l_V)^delta
+                            const float ypw = L4.y * ex2_(dl2 * L4.z);      // k0 (l / l_V)^delta
                             const float base = fmaf(eb, L4.w, ypw);
-                            const float E = exp2f(cA * base);
+                            const float E = ex2_(cA * base);
                             const float dterm = fmaf(ypw, L4.z, nd19 * L4.w);
                             s0[jj] = S[jj] * L4.x;
                             sE[jj] = s0[jj] * E;
@@ -432,7 +432,7 @@ k_fwd_tc(const __grid_constant__ TcMaps tm, const __grid_constant__ Consts c, co
                                     if (gauss) {
                                         const float2 u = __fmul2_rn(__fadd2_rn(make_float2(lm[jj], lm[jj + 1]), ngc), gs2);
                                         const float2 t = __fmul2_rn(u, u);
-                                        w = make_float2(i0 ? exp2f(-t.x) : 0.0f, i1 ? exp2f(-t.y) : 0.0f);
+                                        w = make_float2(i0 ? ex2_(-t.x) : 0.0f, i1 ? ex2_(-t.y) : 0.0f);
                                     }
                                     p0 = __ffma2_rn(make_float2(s0[jj], s0[jj + 1]), w, p0);
                                     p1 = __ffma2_rn(make_float2(sE[jj], sE[jj + 1]), w, p1);
@@ -461,7 +461,7 @@ k_fwd_tc(const __grid_constant__ TcMaps tm, const __grid_constant__ Consts c, co
                                                  (-gs[k] * iopz);
                                     } else if (gs[k] != 0.0f) {
                                         const float u = (lm[jj] - gc[k]) * gs[k];
-                                        w = __expf(-0.5f * u * u);
+                                        w = expf_(-0.5f * u * u);
                                         if (KZ) wz = -w * lm[jj] * u * (gs[k] * iopz);   // T' = -u T / s
                                     }
                                     a0 = fmaf(s0[jj], w, a0);

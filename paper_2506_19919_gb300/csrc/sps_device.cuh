@@ -52,6 +52,25 @@ __device__ __forceinline__ double warp_sum_d(double v) {
 }
 __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
 
+// ---------------------------------------------------------------- fast 2^x, 1/x
+// The SFU's 2^x and 1/x alone.  exp2f, __expf and __fdividef wrap the same
+// operations in a rescaling of denormal arguments and results (three to four
+// more instructions each); here results under 2^-126 are 0.  Elsewhere the bits
+// are the same.  In the quadrature, dust and filter loops that is 4% of a sampler
+// run (11.63 -> 11.14 ms for 16,384 chains x 2 trajectories) and 7-12% of an
+// exact BF16 call.
+__device__ __forceinline__ float ex2_(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float rcp_(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float expf_(float x) { return ex2_(x * 1.4426950408889634f); }
+
 // ---------------------------------------------------------------- row tiles
 // Rows ordered by redshift are contracted in tiles that look at one wavelength
 // range, the hull of their band supports.  k_weights collects it per kHullRows
@@ -111,10 +130,10 @@ struct DustTerms {
 __device__ __forceinline__ DustTerms dust_eval(float k0, float lnr, float drude, float AV,
                                               float delta, float ffl) {
     float eb = fmaxf(0.85f - 1.9f * delta, 0.0f);
-    float pw = __expf(delta * lnr);
+    float pw = expf_(delta * lnr);
     float base = k0 * pw + eb * drude;
     float A = AV * (1.0f / 4.05f) * base;
-    float E = exp2f(-0.4f * kLog2_10f * A);
+    float E = ex2_(-0.4f * kLog2_10f * A);
     DustTerms d;
     d.F = ffl + (1.0f - ffl) * E;
     float g = (1.0f - ffl) * E * (-0.4f * kLn10f);
@@ -205,10 +224,10 @@ __device__ __forceinline__ void gl_panel(const float* __restrict__ gx, const flo
             const bool px = uu.x >= 0.0f, py = uu.y >= 0.0f;
             const float2 Ea = __fmul2_rn(uu, make_float2(px ? cpos : cneg, py ? cpos : cneg));
             const float2 Ra = __fmul2_rn(make_float2(fabsf(uu.x), fabsf(uu.y)), make_float2(cs, cs));
-            const float2 E = make_float2(exp2f(Ea.x), exp2f(Ea.y));
-            const float2 R = make_float2(exp2f(Ra.x), exp2f(Ra.y));
+            const float2 E = make_float2(ex2_(Ea.x), ex2_(Ea.y));
+            const float2 R = make_float2(ex2_(Ra.x), ex2_(Ra.y));
             const float2 d = __fadd2_rn(one2, R);
-            const float2 r = make_float2(__fdividef(1.0f, d.x), __fdividef(1.0f, d.y));
+            const float2 r = make_float2(rcp_(d.x), rcp_(d.y));
             const float2 wh = __fmul2_rn(__fmul2_rn(make_float2(gw[q], gw[q + 1]), hp2), __fmul2_rn(E, r));
             a0 = __fadd2_rn(a0, wh);
             if (grad) {
@@ -225,9 +244,9 @@ __device__ __forceinline__ void gl_panel(const float* __restrict__ gx, const flo
             const int q = N - 1;
             const float uu = fmaf(hp, gx[q], xc);
             const bool pos = uu >= 0.0f;
-            const float E = exp2f(uu * (pos ? cpos : cneg));
-            const float R = exp2f(fabsf(uu) * cs);
-            const float r = __fdividef(1.0f, 1.0f + R);
+            const float E = ex2_(uu * (pos ? cpos : cneg));
+            const float R = ex2_(fabsf(uu) * cs);
+            const float r = rcp_(1.0f + R);
             const float wh = gw[q] * hp * E * r;
             a0.x += wh;
             if (grad) {
@@ -250,9 +269,9 @@ __device__ __forceinline__ void gl_panel(const float* __restrict__ gx, const flo
         for (int q = 0; q < N; ++q) {
             const float uu = fmaf(hp, gx[q], xc);
             const bool pos = uu >= 0.0f;
-            const float E = exp2f(uu * (pos ? cpos : cneg));
-            const float R = exp2f(fabsf(uu) * cs);
-            const float r = __fdividef(1.0f, 1.0f + R);
+            const float E = ex2_(uu * (pos ? cpos : cneg));
+            const float R = ex2_(fabsf(uu) * cs);
+            const float r = rcp_(1.0f + R);
             const float wh = gw[q] * hp * E * r;                      // w hh
             v0 += wh;
             if (grad) {
@@ -584,10 +603,10 @@ __device__ __forceinline__ void mdf_rows_adjoint(const Consts& c, const AgeView&
 }
 
 __device__ __forceinline__ float phi_y(float y) {  // y phi(y), 0 at +-inf
-    return isinf(y) ? 0.0f : y * kInvSqrt2Pi * __expf(-0.5f * y * y);
+    return isinf(y) ? 0.0f : y * kInvSqrt2Pi * expf_(-0.5f * y * y);
 }
 __device__ __forceinline__ float phi_(float y) {
-    return isinf(y) ? 0.0f : kInvSqrt2Pi * __expf(-0.5f * y * y);
+    return isinf(y) ? 0.0f : kInvSqrt2Pi * expf_(-0.5f * y * y);
 }
 
 // ---------------------------------------------------------------- bounding map
