@@ -454,12 +454,44 @@ __global__ void k_zscatter(const Galaxies g, const int32_t* __restrict__ gal_idx
     perm[pos] = (int32_t)row;
     pos_of[row] = pos;
 }
+// The order of few rows in one launch: every row's position is the number of
+// rows before it in (z, row), counted against the keys in shared memory.  Also
+// zeroes the `extra` ints at `zero`.
+constexpr int kZFew = 1024;
+__global__ void __launch_bounds__(kZFew) k_zorder_few(const Galaxies g, const int32_t* __restrict__ gal_idx, int n,
+                                                      int32_t* __restrict__ perm, int32_t* __restrict__ pos_of,
+                                                      int32_t* __restrict__ zero, int extra) {
+    __shared__ __align__(16) float key[kZFew];
+    const int t = threadIdx.x;
+    float z = INFINITY;
+    if (t < n) {
+        const int64_t gi = gal_idx ? (int64_t)gal_idx[t] : t;
+        z = (gi >= 0 && gi < g.n) ? g.z[gi] : 0.0f;
+    }
+    key[t] = z;
+    for (int i = t; i < extra; i += blockDim.x) zero[i] = 0;
+    __syncthreads();
+    if (t >= n) return;
+    int r = 0;
+    for (int j = 0; j < n; j += 4) {
+        const float4 k = *reinterpret_cast<const float4*>(key + j);
+        r += (k.x < z || (k.x == z && j < t)) + (k.y < z || (k.y == z && j + 1 < t)) +
+             (k.z < z || (k.z == z && j + 2 < t)) + (k.w < z || (k.w == z && j + 3 < t));
+    }
+    perm[r] = t;
+    pos_of[t] = r;
+}
 }  // namespace
 
 cudaError_t launch_zsort(const Galaxies& g, const int32_t* gal_idx, int64_t n, int32_t* perm,
                          int32_t* pos_of, int32_t* counts, cudaStream_t s, int64_t extra) {
     if (n <= 0) return cudaSuccess;
     static_assert(kZBuckets == 2 * 1024, "scan layout");
+    if (n <= kZFew) {          // one launch instead of four
+        k_zorder_few<<<1, (unsigned)((n + 31) / 32 * 32), 0, s>>>(g, gal_idx, (int)n, perm, pos_of, counts + kZBuckets,
+                                                                  (int)extra);
+        return cudaGetLastError();
+    }
     cudaError_t e = cudaMemsetAsync(counts, 0, sizeof(int32_t) * (size_t)(kZBuckets + extra), s);
     if (e != cudaSuccess) return e;
     const unsigned blocks = (unsigned)((n + 255) / 256);
