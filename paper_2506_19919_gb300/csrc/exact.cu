@@ -24,49 +24,49 @@ __device__ __forceinline__ uint16_t f_to_bf16(float f) {
 }
 
 // ---------------------------------------------------------------- weights
-__global__ void __launch_bounds__(32 * kWarpsApprox)
-k_weights(const __grid_constant__ Consts c, const Grid grid, const Galaxies g,
-          const float* __restrict__ theta, const int32_t* __restrict__ gal_idx, int64_t n,
-          int bf16, float* __restrict__ W32, uint16_t* __restrict__ Wbf,
-          const int32_t* __restrict__ pos_of, float* __restrict__ W32lo, float* __restrict__ keep,
-          uint32_t* __restrict__ hull) {
-    __shared__ RowScratch scratch[kWarpsApprox];
+// W rows of the exact path, one row per warp: SFH, burst and MDF weights, then
+// W_k = w_i q_j as FP32, its TF32 halves, or BF16 scaled by 2^{e_i}.  Bound by
+// the latency of the quadrature's exponentials and of the row's serial chain:
+// what a warp keeps is cut to 5.8 KB of shared memory and 80 registers (24
+// warps per SM), the bin edges are staged in shared memory (a lane-indexed read
+// of kernel parameters is taken lane by lane), and the warps of a block take
+// their rows after one barrier, so that they share the instruction cache.
+// 100,000 rows, BF16, with the arrays kept for the gradient: 398 us, 507 with four
+// rows per block, 9.6 KB a row and the edges in parameter memory.
+constexpr int kRowWarps = 8;           // warps per block of the row kernels
+struct WeightsWork {
+    float m[kMaxAges], dm0[kMaxAges], dm1[kMaxAges], dm2[kMaxAges], pi[kMaxAges], w[kMaxAges];
+    float q[kMaxMets];
+    float th[SPS_NPARAM];
+    PanelScratch ps;
+};
+template <bool kNonsep>
+__global__ void __launch_bounds__(32 * kRowWarps, 3)
+k_weights(const __grid_constant__ Consts c, const Grid grid, const Galaxies g, const float* __restrict__ theta,
+          const int32_t* __restrict__ gal_idx, int64_t n, int bf16, float* __restrict__ W32,
+          uint16_t* __restrict__ Wbf, const int32_t* __restrict__ pos_of, float* __restrict__ W32lo,
+          float* __restrict__ keep, uint32_t* __restrict__ hull) {
+    __shared__ WeightsWork work[kRowWarps];
+    __shared__ EdgeTables et;
+    extern __shared__ float qms[];         // kNonsep: per warp, q_ij of the row [K]
     const int warp = threadIdx.x >> 5, lane = lane_id();
-    RowScratch& s = scratch[warp];
-    for (int64_t row = (int64_t)blockIdx.x * kWarpsApprox + warp; row < n;
-         row += (int64_t)gridDim.x * kWarpsApprox) {
+    WeightsWork& s = work[warp];
+    float* qm = kNonsep ? qms + warp * (kKTileMax * 32) : nullptr;
+    const AgeView view{s.m, s.dm0, s.dm1, s.dm2, s.pi, s.w, nullptr, s.q, nullptr, &s.ps, et.age, et.lgz};
+    stage_edges(c, et);
+    const int A = c.n_age, Zn = c.n_met;
+    const int64_t per_round = (int64_t)gridDim.x * kRowWarps;
+    const int64_t rounds = (n + per_round - 1) / per_round;
+    for (int64_t rd = 0; rd < rounds; ++rd) {
+        __syncthreads();
+        const int64_t row = (rd * gridDim.x + blockIdx.x) * kRowWarps + warp;
+        if (row >= n) continue;
         const int64_t gi = gal_idx ? (int64_t)gal_idx[row] : row;
-        RowParams p;
-        load_params(c, theta + row * SPS_NPARAM, false, p);
-        if (gi < 0 || gi >= g.n) p.finite = false;
-        if (p.finite) {
-            // with keep (a gradient follows): the derivative integrals too, and the
-            // arrays the adjoint needs are kept for it (m and w are the same
-            // either way: the derivatives are separate accumulators)
-            const double M = age_met_weights(c, s, g.bins + (size_t)gi * c.n_age, g.lnT[gi], g.lT10[gi], p,
-                                             keep != nullptr);
-            if (keep) {
-                const int A = c.n_age;
-                float* kr = keep + row * keep_stride(c);
-                if (lane == 0) *reinterpret_cast<double*>(kr) = M;
-                float* ka = kr + 2;
-                for (int i = lane; i < A; i += 32) {
-                    ka[i] = s.m[i];
-                    ka[A + i] = s.dm[0][i];
-                    ka[2 * A + i] = s.dm[1][i];
-                    ka[3 * A + i] = s.dm[2][i];
-                    ka[4 * A + i] = s.pi[i];
-                    ka[5 * A + i] = s.w[i];
-                }
-                if (lane < c.n_met) ka[6 * A + lane] = s.q[lane];
-            }
-        } else {
-            for (int i = lane; i < c.n_age; i += 32) s.w[i] = __int_as_float(0x7fc00000);
-            if (lane < c.n_met) s.q[lane] = 1.0f;
-            __syncwarp();
-        }
+        const float xk = (lane < SPS_NPARAM) ? theta[row * SPS_NPARAM + lane] : 0.0f;
+        const bool in = gi >= 0 && gi < g.n;
+        const bool ok = __all_sync(kFull, isfinite(xk)) && in;
         const int64_t wr = pos_of ? (int64_t)pos_of[row] : row;
-        if (hull && gi >= 0 && gi < g.n) {             // this row's part of its tile's hull (see row_hull)
+        if (hull && in) {                              // this row's part of its tile's hull (see row_hull)
             const int2 sp = lane < c.n_band ? g.support[gi * c.n_band + lane] : make_int2(0, 0);
             const bool any = sp.x < sp.y;
             const uint32_t below = __reduce_max_sync(kFull, any ? (uint32_t)(c.n_lam - sp.x) : 0u);
@@ -76,11 +76,39 @@ k_weights(const __grid_constant__ Consts c, const Grid grid, const Galaxies g,
                 atomicMax(hull + 2 * (wr / kHullRows) + 1, above);
             }
         }
-        const bool nonsep = c.mdf_age != 0 && p.finite;
-        if (nonsep) mdf_rows_fill(c, c.lgz_edge, p.th[7], p.th[8], s.u.kbuf);
+        if (lane < SPS_NPARAM) s.th[lane] = xk;
+        __syncwarp();
+        if (ok) {
+            // with keep (a gradient follows): the derivative integrals too, and the
+            // arrays the adjoint needs are kept for it
+            age_met_parts<true>(c, view, g.bins + (size_t)gi * A, g.lnT[gi], g.lT10[gi], s.th, keep != nullptr);
+            __syncwarp();
+            const double M = warp_sum_d(mass_partial(c, view));
+            age_weights(c, view, s.th, M);
+            if (keep) {
+                float* kr = keep + row * keep_stride(c);
+                if (lane == 0) *reinterpret_cast<double*>(kr) = M;
+                float* ka = kr + 2;
+                for (int i = lane; i < A; i += 32) {
+                    ka[i] = s.m[i];
+                    ka[A + i] = s.dm0[i];
+                    ka[2 * A + i] = s.dm1[i];
+                    ka[3 * A + i] = s.dm2[i];
+                    ka[4 * A + i] = s.pi[i];
+                    ka[5 * A + i] = s.w[i];
+                }
+                if (lane < Zn) ka[6 * A + lane] = s.q[lane];
+            }
+            if (kNonsep) mdf_rows_fill(c, et.lgz, s.th[7], s.th[8], qm);
+        } else {
+            for (int i = lane; i < A; i += 32) s.w[i] = __int_as_float(0x7fc00000);
+            if (lane < Zn) s.q[lane] = 1.0f;
+            if (kNonsep)
+                for (int k = lane; k < c.K; k += 32) qm[k] = 1.0f;
+            __syncwarp();
+        }
         // W_k = w_i q_j, k = i Zn + j: a lane writes the pair (k, k + 1) for
         // k = 2 lane + 64 t (k_pad is even), with (i, j) of k kept incrementally
-        const int Zn = c.n_met;
         int k = 2 * lane;
         int i = k / Zn, j = k - i * Zn;
         const int di = 64 / Zn, dj = 64 - di * Zn;
@@ -91,12 +119,12 @@ k_weights(const __grid_constant__ Consts c, const Grid grid, const Galaxies g,
                 ++i1;
             }
             float v0 = 0.0f, v1 = 0.0f;
-            if (k < c.K) v0 = s.w[i] * (nonsep ? s.u.kbuf[k] : s.q[j]);
-            if (k + 1 < c.K) v1 = s.w[i1] * (nonsep ? s.u.kbuf[k + 1] : s.q[j1]);
+            if (k < c.K) v0 = s.w[i] * (kNonsep ? qm[k] : s.q[j]);
+            if (k + 1 < c.K) v1 = s.w[i1] * (kNonsep ? qm[k + 1] : s.q[j1]);
             const int64_t o = wr * c.k_pad + k;
             if (bf16) {
-                const float b0 = k < c.K ? v0 * grid.row_scale[i] : 0.0f;
-                const float b1 = k + 1 < c.K ? v1 * grid.row_scale[i1] : 0.0f;
+                const float2 sc = *reinterpret_cast<const float2*>(grid.col_scale + k);   // 2^{e_i}, 0 past K
+                const float b0 = v0 * sc.x, b1 = v1 * sc.y;
                 *reinterpret_cast<uint32_t*>(Wbf + o) = (uint32_t)f_to_bf16(b0) | ((uint32_t)f_to_bf16(b1) << 16);
             } else if (W32lo) {                        // 3xTF32 operand halves
                 float h0, l0, h1, l1;
@@ -392,6 +420,130 @@ k_exact_grad(const __grid_constant__ Consts c, const Galaxies g, const float* __
     }
 }
 
+// k_exact_grad for the separable model with Zn <= kZnReg: lane i takes age rows
+// i, i + 32, ... of Wbar in 16-byte loads straight from memory, wbar_i = sum_j
+// Wbar_ij q_j and its share of qbar_j = sum_i w_i Wbar_ij in registers, and the
+// lanes' shares are added up through shared memory; k_exact_grad stages the row
+// in shared memory and sums each qbar_j in one lane over all ages.  Blocks in
+// step and edges in shared memory as in k_weights.
+// 100,000 rows: 206 us against 317.
+struct GradWork {
+    float m[kMaxAges], dm0[kMaxAges], dm1[kMaxAges], dm2[kMaxAges], pi[kMaxAges], wb[kMaxAges];
+    float qb[kMaxMets];
+    float th[SPS_NPARAM];
+    float red[32][kZnReg + 1];
+};
+__global__ void __launch_bounds__(32 * kRowWarps, 4)
+k_exact_grad_sep(const __grid_constant__ Consts c, const Galaxies g, const float* __restrict__ theta,
+                 const int32_t* __restrict__ gal_idx, int64_t n, const float* __restrict__ rowinfo,
+                 const float* __restrict__ Wbar, float* __restrict__ grad_out, const float* __restrict__ rowz,
+                 const float* __restrict__ keep, const int32_t* __restrict__ pos_of, int nsplit) {
+    __shared__ GradWork work[kRowWarps];
+    __shared__ EdgeTables et;
+    const int warp = threadIdx.x >> 5, lane = lane_id();
+    GradWork& s = work[warp];
+    const AgeView view{s.m, s.dm0, s.dm1, s.dm2, s.pi, nullptr, s.wb, nullptr, s.qb, nullptr, et.age, et.lgz};
+    stage_edges(c, et);
+    const int A = c.n_age, Zn = c.n_met;
+    const int NG = rowz ? SPS_NPARAM + 1 : SPS_NPARAM;       // with rowz: d/dz last
+    const int64_t per_round = (int64_t)gridDim.x * kRowWarps;
+    const int64_t rounds = (n + per_round - 1) / per_round;
+    for (int64_t rd = 0; rd < rounds; ++rd) {
+        __syncthreads();
+        const int64_t row = (rd * gridDim.x + blockIdx.x) * kRowWarps + warp;
+        if (row >= n) continue;
+        const int64_t gi = gal_idx ? (int64_t)gal_idx[row] : row;
+        const float xk = (lane < SPS_NPARAM) ? theta[row * SPS_NPARAM + lane] : 0.0f;
+        if (!(__all_sync(kFull, isfinite(xk)) && gi >= 0 && gi < g.n)) {
+            if (lane < NG) grad_out[row * NG + lane] = __int_as_float(0x7fc00000);
+            continue;
+        }
+        if (lane < SPS_NPARAM) s.th[lane] = xk;
+        const float* kr = keep + row * keep_stride(c);           // the weights kernel's arrays of this row
+        const double M = *reinterpret_cast<const double*>(kr);
+        const float* ka = kr + 2;
+        const float* wr = Wbar + (pos_of ? (int64_t)pos_of[row] : row) * c.k_pad;
+        float q[kZnReg], U[kZnReg];
+#pragma unroll
+        for (int j = 0; j < kZnReg; ++j) {
+            q[j] = j < Zn ? __ldg(ka + 6 * A + j) : 0.0f;
+            U[j] = 0.0f;
+        }
+#pragma unroll 2
+        for (int i = lane; i < A; i += 32) {
+            float v[kZnReg];
+            load_row(wr + i * Zn, Zn, v);
+            for (int p = 1; p < nsplit; ++p) {
+                float x[kZnReg];
+                load_row(wr + (int64_t)p * n * c.k_pad + i * Zn, Zn, x);
+#pragma unroll
+                for (int j = 0; j < kZnReg; ++j) v[j] += x[j];
+            }
+            const float wi = ka[5 * A + i];
+            s.m[i] = ka[i];
+            s.dm0[i] = ka[A + i];
+            s.dm1[i] = ka[2 * A + i];
+            s.dm2[i] = ka[3 * A + i];
+            s.pi[i] = ka[4 * A + i];
+            float a = 0.0f;
+#pragma unroll
+            for (int j = 0; j < kZnReg; ++j) {
+                a = fmaf(v[j], q[j], a);
+                U[j] = fmaf(v[j], wi, U[j]);
+            }
+            s.wb[i] = a;
+        }
+#pragma unroll
+        for (int j = 0; j < kZnReg; ++j) s.red[lane][j] = U[j];
+        __syncwarp();
+        {
+            const int j = lane & 15, h = lane >> 4;
+            float a = 0.0f;
+            if (j < kZnReg) {
+#pragma unroll 8
+                for (int r = 0; r < 16; ++r) a += s.red[16 * h + r][j];
+            }
+            a += __shfl_down_sync(kFull, a, 16);
+            if (lane < Zn) s.qb[lane] = a;
+        }
+        __syncwarp();
+        float gr[SPS_NPARAM];
+#pragma unroll
+        for (int k = 0; k < SPS_NPARAM; ++k) gr[k] = 0.0f;
+        const float4 ri = *reinterpret_cast<const float4*>(rowinfo + row * 4);
+        gr[0] = ri.x;
+        gr[9] = ri.y;
+        gr[10] = ri.z;
+        gr[11] = ri.w;
+        age_met_adjoint(c, view, g.lT10[gi], M, s.th, gr);
+        float gzt = 0.0f;          // d log L / dz through t_obs (age bins, M, burst clipping)
+        if (rowz)
+            gzt = rowz[row] + g.dtdz[gi] * tobs_adjoint(c, view, g.bins + (size_t)gi * A, g.lnT[gi], g.lT10[gi], M,
+                                                         s.th);
+        float out = gr[0];
+#pragma unroll
+        for (int k = 1; k < SPS_NPARAM; ++k)
+            if (lane == k) out = gr[k];
+        if (lane == SPS_NPARAM) out = gzt;
+        if (lane < NG) grad_out[row * NG + lane] = out;
+        __syncwarp();
+    }
+}
+
+// Blocks of a row kernel: persistent, as many as are resident.
+template <class K>
+cudaError_t row_blocks(K kern, size_t smem, int64_t n, int& blocks) {
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaError_t e;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kRowWarps, smem)) != cudaSuccess) return e;
+    const int64_t need = (n + kRowWarps - 1) / kRowWarps;
+    const int64_t most = (int64_t)(per_sm > 0 ? per_sm : 1) * sms;
+    blocks = (int)(need < most ? need : most);
+    return cudaSuccess;
+}
+
 int blocks_rows(int64_t rows, int per_block) {
     int64_t b = (rows + per_block - 1) / per_block;
     if (b > 152LL * 64) b = 152LL * 64;
@@ -405,9 +557,19 @@ cudaError_t launch_exact_weights(const Consts& c, const Grid& grid, const Galaxi
                                  float* W32, uint16_t* Wbf, cudaStream_t s, const int32_t* pos_of,
                                  float* W32lo, float* keep, uint32_t* hull) {
     if (n <= 0) return cudaSuccess;
-    k_weights<<<blocks_rows(n, kWarpsApprox), 32 * kWarpsApprox, 0, s>>>(c, grid, g, theta, gal_idx,
-                                                                         n, bf16, W32, Wbf, pos_of, W32lo,
-                                                                         keep, hull);
+    int blocks = 0;
+    cudaError_t e;
+    if (c.mdf_age) {
+        const size_t smem = sizeof(float) * kKTileMax * 32 * kRowWarps;
+        e = cudaFuncSetAttribute(k_weights<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess || (e = row_blocks(k_weights<true>, smem, n, blocks)) != cudaSuccess) return e;
+        k_weights<true><<<blocks, 32 * kRowWarps, smem, s>>>(c, grid, g, theta, gal_idx, n, bf16, W32, Wbf, pos_of,
+                                                             W32lo, keep, hull);
+    } else {
+        if ((e = row_blocks(k_weights<false>, 0, n, blocks)) != cudaSuccess) return e;
+        k_weights<false><<<blocks, 32 * kRowWarps, 0, s>>>(c, grid, g, theta, gal_idx, n, bf16, W32, Wbf, pos_of,
+                                                           W32lo, keep, hull);
+    }
     return cudaGetLastError();
 }
 
@@ -528,6 +690,14 @@ cudaError_t launch_exact_grad(const Consts& c, const Galaxies& g, const float* t
                               const float* Wbar, float* grad_out, cudaStream_t s, const float* rowz,
                               const float* keep, const int32_t* pos_of, int nsplit) {
     if (n <= 0) return cudaSuccess;
+    if (!c.mdf_age && c.n_met <= kZnReg && keep) {
+        int blocks = 0;
+        const cudaError_t e = row_blocks(k_exact_grad_sep, 0, n, blocks);
+        if (e != cudaSuccess) return e;
+        k_exact_grad_sep<<<blocks, 32 * kRowWarps, 0, s>>>(c, g, theta, gal_idx, n, rowinfo, Wbar, grad_out, rowz, keep,
+                                                           pos_of, nsplit);
+        return cudaGetLastError();
+    }
     k_exact_grad<<<blocks_rows(n, kWarpsApprox), 32 * kWarpsApprox, 0, s>>>(c, g, theta, gal_idx, n,
                                                                             rowinfo, Wbar, grad_out, rowz, keep,
                                                                             pos_of, nsplit);

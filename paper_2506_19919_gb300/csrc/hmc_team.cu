@@ -25,7 +25,6 @@ namespace sps {
 
 namespace {
 
-constexpr int kZnReg = 12;   // metallicity bins held in registers (Zn <= 12)
 
 template <int CPW>
 struct TeamWork {
@@ -76,12 +75,6 @@ struct TeamWork {
     float nu[CPW][32];                      // uniforms of the subtree's next 32 leaves
 };
 
-// Age and metallicity bin edges of the tables, staged once per block.
-struct EdgeTables {
-    float age[kMaxAges + 1];
-    float lgz[kMaxMets + 1];
-};
-
 template <int CPW>
 __device__ __forceinline__ AgeView age_view(TeamWork<CPW>& t, int ch, const EdgeTables& et) {
     return AgeView{t.m[ch], t.dm0[ch], t.dm1[ch], t.dm2[ch], t.pi[ch], t.w[ch], t.w[ch],
@@ -94,20 +87,6 @@ __device__ __forceinline__ void prefetch_l2(const float* p, uint32_t bytes) {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 constexpr int kAhead = 2;    // bands prefetched ahead
-
-// Row i of a band's c_SSP table: Zn consecutive floats.
-__device__ __forceinline__ void load_row(const float* __restrict__ p, int Zn, float* cv) {
-    if (Zn == 12) {
-        const float4* v = reinterpret_cast<const float4*>(p);
-        float4 a = v[0], b = v[1], c = v[2];
-        cv[0] = a.x; cv[1] = a.y; cv[2] = a.z; cv[3] = a.w;
-        cv[4] = b.x; cv[5] = b.y; cv[6] = b.z; cv[7] = b.w;
-        cv[8] = c.x; cv[9] = c.y; cv[10] = c.z; cv[11] = c.w;
-    } else {
-#pragma unroll
-        for (int j = 0; j < kZnReg; ++j) cv[j] = (j < Zn) ? p[j] : 0.0f;
-    }
-}
 
 // log posterior (unbounded space) and its gradient for every chain of the
 // team at t.x; writes t.lp and t.g.

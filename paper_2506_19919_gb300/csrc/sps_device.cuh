@@ -188,6 +188,31 @@ struct RowScratch {
     }
 };
 
+// Age and metallicity bin edges of the tables, staged once per block.
+struct EdgeTables {
+    float age[kMaxAges + 1];
+    float lgz[kMaxMets + 1];
+};
+__device__ __forceinline__ void stage_edges(const Consts& c, EdgeTables& et) {
+    for (int i = threadIdx.x; i <= c.n_age; i += blockDim.x) et.age[i] = c.log_age_edge[i];
+    for (int i = threadIdx.x; i <= c.n_met; i += blockDim.x) et.lgz[i] = c.lgz_edge[i];
+}
+
+constexpr int kZnReg = 12;   // metallicity bins held in registers (Zn <= 12)
+// An age row of a table with Zn <= kZnReg columns: Zn consecutive floats.
+__device__ __forceinline__ void load_row(const float* __restrict__ p, int Zn, float* cv) {
+    if (Zn == 12) {
+        const float4* v = reinterpret_cast<const float4*>(p);
+        float4 a = v[0], b = v[1], c = v[2];
+        cv[0] = a.x; cv[1] = a.y; cv[2] = a.z; cv[3] = a.w;
+        cv[4] = b.x; cv[5] = b.y; cv[6] = b.z; cv[7] = b.w;
+        cv[8] = c.x; cv[9] = c.y; cv[10] = c.z; cv[11] = c.w;
+    } else {
+#pragma unroll
+        for (int j = 0; j < kZnReg; ++j) cv[j] = (j < Zn) ? p[j] : 0.0f;
+    }
+}
+
 // ---------------------------------------------------------------- SFH bins
 // Panel count ceil(f) clamped to [1, kMaxPanels]; NaN or inf give a bounded
 // count so that no input can index outside the scratch arrays.
