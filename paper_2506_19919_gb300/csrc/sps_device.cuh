@@ -402,22 +402,24 @@ __device__ __forceinline__ void sfh_bins_raw(const Consts& c, const AgeView& v, 
                 v.dm2[i] = v3 * tau;
             }
         }
-        // queue the panels of multi-panel bins: exclusive scan of their counts
+        // queue the panels of multi-panel bins: exclusive scan of their counts (most
+        // groups of 32 bins have none)
         const int nq = (n >= 2) ? n : 0;
-        int incl = nq;
+        if (__any_sync(kFull, nq > 0)) {
+            int incl = nq;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(kFull, incl, o);
-            if (lane >= o) incl += t;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int t = __shfl_up_sync(kFull, incl, o);
+                if (lane >= o) incl += t;
+            }
+            const int st = base + incl - nq;
+            if (nq > 0) {
+                ps.info[i] = make_float4(x0, hp, __int_as_float(st), 0.0f);
+                if (st < kMaxPanels) ps.pmap[st] = (unsigned char)i;
+            }
+            base += __shfl_sync(kFull, incl, 31);
         }
-        const int st = base + incl - nq;
-        if (nq > 0) {
-            ps.info[i] = make_float4(x0, hp, __int_as_float(st), 0.0f);
-            if (st < kMaxPanels) ps.pmap[st] = (unsigned char)i;
-        } else if (i < A) {
-            ps.info[i].z = __int_as_float(-1);       // not queued in this call
-        }
-        base += __shfl_sync(kFull, incl, 31);
+        if (nq == 0 && i < A) ps.info[i].z = __int_as_float(-1);       // not queued in this call
     }
     const int P = min(base, kMaxPanels);
     __syncwarp();
