@@ -1215,10 +1215,14 @@ extern "C" sps_status sps_hmc_run(sps_ctx* ctx, const sps_hmc_config* cfg, const
     // launch shapes: chains of a galaxy per warp (cpw) x warps per block; the
     // grid is persistent (occupancy x SMs) and pulls (galaxy, chain group)
     // items from the queue
-    // first candidate = default; another replaces it only if >3% faster in the probe
+    // the first candidate is the one to beat: another replaces it only if >3% faster
+    // in the probe.  One chain per warp runs 24 warps per SM in 80 registers, two
+    // chains 16 in 128: 16,384 chains x 2 trajectories 9.0 ms against 11.2; two per
+    // warp stays a candidate for tables that do not fit L2, which it reads half as
+    // often, and the shape without a probe
     // an age-dependent MDF runs the one-chain-per-warp variant with the per-age q matrix
     const bool rows = ctx->c.mdf_age != 0;
-    std::vector<std::pair<int, int>> cands = {{1, 8}, {1, 16}};
+    std::vector<std::pair<int, int>> cands = {{1, 8}};
     if (rows) {
         cands = {{1, 4}, {1, 2}, {1, 8}};
     } else if (nuts) {
@@ -1228,10 +1232,9 @@ extern "C" sps_status sps_hmc_run(sps_ctx* ctx, const sps_hmc_config* cfg, const
         cands = {{1, 8}};
         if (C >= 2) cands.push_back({2, 8});
     } else {
-        if (C >= 2) cands.insert(cands.begin(), {{2, 4}, {2, 8}, {2, 16}});
-        if (C >= 4) cands.push_back({4, 8});
+        if (C >= 2) cands.push_back({2, 8});
     }
-    const int cpw0 = cands[0].first;
+    const std::pair<int, int> dflt = (!rows && !nuts && C >= 2) ? std::make_pair(2, 4) : cands[0];
     auto blocks_for = [&](int cpw, int warps, int& blocks) -> cudaError_t {
         int per_sm = 0;
         cudaError_t e = hmc_team_occupancy(cpw, rows, nuts, warps, &per_sm);
@@ -1241,15 +1244,25 @@ extern "C" sps_status sps_hmc_run(sps_ctx* ctx, const sps_hmc_config* cfg, const
     };
     const std::string key = std::to_string(G) + ":" + std::to_string(C) + ":" + std::to_string(nb_max) +
                             (nuts ? ":nuts" : "") + (rows ? ":rows" : "");
-    int cpw = cpw0, warps = cands[0].second, blocks = sms;
+    int cpw = dflt.first, warps = dflt.second, blocks = sms;
+    // chains that all fit at once, one per warp, run that way, spread over the SMs:
+    // a warp with one chain takes 0.57 of the time of one with two
+    int few_blocks = 0;
+    CK(blocks_for(1, rows ? 4 : 8, few_blocks));
+    const bool few = NC <= (int64_t)few_blocks * (rows ? 4 : 8);
     auto it = ctx->tuned.find(key);
     const char* force = std::getenv("SPS_HMC_SHAPE");   // "cpw,warps": fixed launch shape
     int fc = 0, fw = 0;
     if (force && std::sscanf(force, "%d,%d", &fc, &fw) == 2 && (fc == 1 || (!rows && (fc == 2 || fc == 4))) &&
         fc <= std::max(C, 1) && fw >= 1 && fw <= 16) {
         cpw = fc;
-        warps = fw;
+        warps = (fc == 1 && !rows) ? std::min(fw, 8) : fw;
         CK(blocks_for(cpw, warps, blocks));
+    } else if (few) {
+        cpw = 1;
+        warps = (int)std::max<int64_t>(1, std::min<int64_t>((NC + sms - 1) / sms, rows ? 4 : 8));
+        CK(blocks_for(cpw, warps, blocks));
+        blocks = (int)std::min<int64_t>(blocks, (NC + warps - 1) / warps);
     } else if (it != ctx->tuned.end()) {
         cpw = it->second.first / 100;
         warps = it->second.first % 100;
@@ -1297,7 +1310,7 @@ extern "C" sps_status sps_hmc_run(sps_ctx* ctx, const sps_hmc_config* cfg, const
     // (HMC, separable model, an even chain count): the same chains and draws,
     // spread over more warps. SPS_HMC_TAIL=0 keeps one launch.
     int64_t main_end = -1;      // two-chain items of the first launch (< 0: all)
-    int blocks1 = 0;
+    int blocks1 = 0, warps1 = 0;
     {
         const int64_t slots = (int64_t)blocks * warps;
         const int64_t items = G * (int64_t)((C + cpw - 1) / cpw);
@@ -1305,7 +1318,8 @@ extern "C" sps_status sps_hmc_run(sps_ctx* ctx, const sps_hmc_config* cfg, const
         if (!nuts && !rows && cpw == 2 && C % 2 == 0 && !(tv && tv[0] == '0') && items > slots &&
             items % slots != 0 && 4 * (items % slots) < 3 * slots) {
             main_end = items / slots * slots;
-            CK(blocks_for(1, warps, blocks1));
+            warps1 = std::min(warps, 8);     // the one-chain kernel's block limit
+            CK(blocks_for(1, warps1, blocks1));
             if (!ctx->side) {
                 CK(cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking));
                 CK(cudaEventCreateWithFlags(&ctx->fork, cudaEventDisableTiming));
@@ -1333,7 +1347,7 @@ extern "C" sps_status sps_hmc_run(sps_ctx* ctx, const sps_hmc_config* cfg, const
         h2.item0 = 2 * main_end;      // one-chain items: two per two-chain item
         h2.item_end = G * (int64_t)C;
         e = launch_hmc_team(1, rows, c, ctx->gal(), h2, x0, mo, sg, mk, ord, so, acc, epo, dv, nev, sto,
-                            ctx->queue.as<int>() + 1, cmet, blocks1, warps, ctx->side);
+                            ctx->queue.as<int>() + 1, cmet, blocks1, warps1, ctx->side);
         if (e != cudaSuccess) return e;
         if ((e = cudaEventRecord(ctx->join, ctx->side)) != cudaSuccess) return e;
         return cudaStreamWaitEvent(s, ctx->join, 0);

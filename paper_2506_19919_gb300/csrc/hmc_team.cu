@@ -1100,9 +1100,13 @@ __host__ __device__ constexpr size_t team_stride() {
 // Persistent kernel: each warp is a team working through the queue of
 // (galaxy, chain group) items; the warps of a block advance one evaluation per
 // pass together (one block barrier per pass), so that they run the same code
-// at the same time and share the instruction cache.
+// at the same time and share the instruction cache.  One chain per warp takes
+// three blocks of eight warps per SM (80 registers; the state of 24 warps is what
+// shared memory holds): the kernel waits on the latency of its exponentials and
+// reductions, and 24 one-chain warps hide more of it than 16 two-chain ones save
+// in table loads (16,384 chains x 2 trajectories, 9.03 ms against 11.16).
 template <int CPW, bool kNonsep, bool kNuts>
-__global__ void __launch_bounds__(512, 1)
+__global__ void __launch_bounds__(CPW == 1 && !kNonsep ? 256 : 512, CPW == 1 && !kNonsep ? 3 : 1)
 k_hmc_team(const __grid_constant__ Consts c, const Galaxies g, const HmcParams hp,
            const float* __restrict__ theta0, const float* __restrict__ mag_obs,
            const float* __restrict__ sigma, const uint32_t* __restrict__ mask,
