@@ -32,7 +32,7 @@ constexpr int kFwdStages = 4;    // BF16 ring depth
 constexpr int kFwdBNtf = 128;
 constexpr int kFwdStagesTf = 3;  // four 16 KB tiles per stage
 constexpr int kAdjBN = 224;      // K = 1344 = 6 x 224: each 128-row block streams V six times
-constexpr int kAdjStages = 5;    // BF16 ring depth (TF32: 2)
+constexpr int kAdjStages = 4;    // BF16 ring depth (TF32: 2)
 constexpr uint32_t kTmemCols = 512;
 // Forward epilogue: per warp, the wavelength constants (lamc, lam) of the
 // 32-column chunk being processed, staged in shared memory after the control
