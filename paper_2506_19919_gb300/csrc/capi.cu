@@ -662,12 +662,13 @@ static sps_status run_exact(sps_ctx* ctx, const float* theta, const int32_t* gid
                                 pos_of, tf ? ctx->Wlo.as<float>() : nullptr, keep, hull));
         if (tc) {
             TcMaps tm;
+            const uint32_t bn = (uint32_t)tc_fwd_columns(c, tf);
             const bool ok = tf ? (make_tmap_f32(&tm.a[0], ctx->W.p, c.k_pad, m, c.k_pad, 128) &&
                                   make_tmap_f32(&tm.a[1], ctx->Wlo.p, c.k_pad, m, c.k_pad, 128) &&
-                                  make_tmap_f32(&tm.b[0], ctx->ssp_t_hi.p, c.k_pad, c.n_lam, c.k_pad, 128) &&
-                                  make_tmap_f32(&tm.b[1], ctx->ssp_t_lo.p, c.k_pad, c.n_lam, c.k_pad, 128))
+                                  make_tmap_f32(&tm.b[0], ctx->ssp_t_hi.p, c.k_pad, c.n_lam, c.k_pad, bn) &&
+                                  make_tmap_f32(&tm.b[1], ctx->ssp_t_lo.p, c.k_pad, c.n_lam, c.k_pad, bn))
                                : (make_tmap_bf16(&tm.a[0], ctx->W.p, c.k_pad, m, c.k_pad, 128) &&
-                                  make_tmap_bf16(&tm.b[0], ctx->ssp_t_bf.p, c.k_pad, c.n_lam, c.k_pad, 256));
+                                  make_tmap_bf16(&tm.b[0], ctx->ssp_t_bf.p, c.k_pad, c.n_lam, c.k_pad, bn));
             if (!ok) return fail(SPS_E_CUDA, "tensor map encoding failed");
             if (!tf) tm.a[1] = tm.a[0], tm.b[1] = tm.b[0];
             CK(launch_fwd_tc(tm, tf, c, grid, gv, th, gi, perm, hull, m, ctx->cJ.as<float>(), fsplit, terr, s, cJz));

@@ -151,7 +151,7 @@ int adj_tpc(const Consts& c, int64_t n) {
 // (100,000 rows in 3 parts: 2.04 ms against 1.96).
 int tc_fwd_split(const Consts& c, int64_t n, bool tf) {
     const int64_t mt = (n + kTM - 1) / kTM;
-    const int bn = tf ? kFwdBNtf : kFwdBN;
+    const int bn = tc_fwd_columns(c, tf);
     const int most = std::min(24, (c.n_lam + bn - 1) / bn);
     return (int)std::max<int64_t>(1, std::min<int64_t>(kSms / mt, most));
 }
@@ -163,10 +163,7 @@ int tc_adj_split(const Consts& c, int64_t n) {
     return (int)std::max<int64_t>(1, std::min<int64_t>(kSms / blocks, 8));
 }
 
-size_t tc_fwd_smem(bool tf) {
-    return (tf ? Ring<kFwdBNtf, kFwdStagesTf, true>::kBytes : Ring<kFwdBN, kFwdStages, false>::kBytes) + 256 +
-           kFwdConstBytes + 1024;
-}
+int tc_fwd_columns(const Consts& c, bool tf) { return fwd_shape(c.n_band, tf).bn; }
 size_t tc_adj_smem(bool tf) {
     return (tf ? Ring<kAdjBN, 2, true>::kBytes : Ring<kAdjBN, kAdjStages, false>::kBytes) + 256 +
            4 * 32 * kTrPitch * sizeof(float) + 1024;

@@ -20,17 +20,31 @@ namespace {
 constexpr int kTM = 128;       // rows per tile (MMA M)
 constexpr int kRowBytes = 128; // one k-block row: 64 BF16 or 32 FP32 (128-byte swizzle)
 constexpr int kThreadsTC = 192;   // adjoint: TMA warp, MMA warp, 4 epilogue warps
-constexpr int kFwdGroupBands = 8; // forward: bands per epilogue warp
 constexpr int kFwdMaxEpiWarps = 16;
-constexpr int kFwdBN = 256;
-constexpr int kFwdStages = 4;    // BF16 ring depth
-// 3xTF32 forward: 128-column tiles, each with two TMEM accumulators (the
+// 3xTF32 forward: 128- or 96-column tiles, each with two TMEM accumulators (the
 // hi x hi product, and the hi x lo + lo x hi corrections, added in FP32 in the
 // epilogue), so that the large accumulator takes a third of the additions:
 // the tensor core's FP32 accumulation loses a fraction of an ulp per addition
 // in one direction, which over 3 x 168 additions left fluxes ~1.5e-5 low
-constexpr int kFwdBNtf = 128;
-constexpr int kFwdStagesTf = 3;  // four 16 KB tiles per stage
+// Forward shapes.  The epilogue warps hold a group of bands in registers and
+// take a part of the tile's columns.  Up to six bands: three parts, 12 warps at
+// 128 registers, tiles of 192 columns (96 for 3xTF32); the epilogue is bound by
+// the latency of its exponentials and TMEM loads (100,000 rows, six bands, BF16
+// photometry 1.41 ms a call; two parts, 8 warps at 168 registers and 256 columns
+// 1.51; four parts, 16 warps at 96 registers 1.91).  Seven to 16 bands: eight per
+// warp, 8 warps at 168 registers, 256 (128) columns; more bands: eight per warp
+// in three or four groups.
+struct FwdShape {
+    int bands, groups, parts, bn;
+};
+inline FwdShape fwd_shape(int n_band, bool tf) {
+    if (n_band <= 6) return FwdShape{6, 1, 3, tf ? 96 : 192};
+    const int groups = (n_band + 7) / 8;                   // <= 4 (n_band <= 32)
+    return FwdShape{8, groups, groups == 1 ? 2 : 1, tf ? 128 : 256};
+}
+// Ring depth of a forward shape (the 192-column stages are smaller).
+template <int BN, bool TF>
+constexpr int kFwdStages = TF ? 3 : BN == 192 ? 5 : 4;
 constexpr int kAdjBN = 224;      // K = 1344 = 6 x 224: each 128-row block streams V six times
 constexpr int kAdjStages = 4;    // BF16 ring depth (TF32: 2)
 constexpr uint32_t kTmemCols = 512;
@@ -225,26 +239,27 @@ __device__ __forceinline__ uint8_t* carve(unsigned char* raw, Ctl*& ctl) {
 }
 
 // ---------------------------------------------------------------- forward
-// Epilogue layout: 4 x n_groups x n_halves warps.  A warp reads the TMEM lane
-// quarter q = (warp id mod 4) (32 rows) of each tile, for the bands of its group (<= 8, held in
-// registers) and, when one group covers all bands, for one half of the tile's
-// columns.  Rows arrive sorted by redshift (perm), so the 32 rows of a warp see
+// Epilogue layout: 4 x n_groups x n_halves warps (fwd_shape).  A warp reads the TMEM lane
+// quarter q = (warp id mod 4) (32 rows) of each tile, for the bands of its group (<= NB, held in
+// registers) and one of n_halves (1, 2 or 3) parts of the tile's columns.  Rows arrive sorted by redshift (perm), so the 32 rows of a warp see
 // nearly the same band supports: a band is visited in a 32-column chunk only if
 // it overlaps the chunk in some lane.
 // KZ also accumulates the redshift derivative of the band weights,
 // wb' = q_n T'((1+z) l_n), into cJz[row][b][2] = sum_n wb' S (1, E).
-template <int MAXT, bool TF, bool KZ = false>
+template <int MAXT, int NB, int BN, bool TF, bool KZ>
 __global__ void __launch_bounds__(MAXT, 1)
 k_fwd_tc(const __grid_constant__ TcMaps tm, const __grid_constant__ Consts c, const Grid grid, const Galaxies g,
          const float* __restrict__ theta, const int32_t* __restrict__ gal_idx,
          const int32_t* __restrict__ perm, const uint32_t* __restrict__ hull, int64_t n, int n_halves,
          float* __restrict__ cJ, int* err, float* __restrict__ cJz) {
-    constexpr int NB = kFwdGroupBands;
     extern __shared__ unsigned char smem_raw[];
     Ctl* ctl;
-    constexpr int BN = TF ? kFwdBNtf : kFwdBN;
-    constexpr int ST = TF ? kFwdStagesTf : kFwdStages;
+    constexpr int ST = kFwdStages<BN, TF>;
     constexpr int ACC = TF ? 2 * BN : BN;          // TMEM columns per buffer
+    // with 12 or 16 epilogue warps (128 or 96 registers) the column groups are a
+    // loop, not unrolled: what the unrolled copies hold in common spilled (20 bands:
+    // 15,000 rows BF16 1.26 ms against 1.31, 4,000 rows 3xTF32 0.78 against 0.86)
+    constexpr int kUnroll = MAXT > 64 + 32 * 8 ? 1 : 4;
     using R = Ring<BN, ST, TF>;
     uint8_t* ring = carve<BN, ST, TF>(smem_raw, ctl);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -316,12 +331,12 @@ k_fwd_tc(const __grid_constant__ TcMaps tm, const __grid_constant__ Consts c, co
         }
         // warp-wide hull of each band's support (lanes without the band excluded):
         // a group is visited for a band if the hull reaches it
-        int hlo[NB], hhi[NB];
+        uint32_t hxy[NB];                          // [lo, hi): lo | hi << 16
 #pragma unroll
         for (int k = 0; k < NB; ++k) {
             const int lo = (int)(sxy[k] & 0xffffu), hi = (int)(sxy[k] >> 16);
-            hlo[k] = (int)__reduce_min_sync(0xffffffffu, (unsigned)(lo < hi ? lo : 0xffff));
-            hhi[k] = (int)__reduce_max_sync(0xffffffffu, (unsigned)(lo < hi ? hi : 0));
+            hxy[k] = __reduce_min_sync(0xffffffffu, (unsigned)(lo < hi ? lo : 0xffff)) |
+                     (__reduce_max_sync(0xffffffffu, (unsigned)(lo < hi ? hi : 0)) << 16);
         }
         bool has_tab = false;                      // a tabulated band in this warp's group
 #pragma unroll
@@ -379,7 +394,7 @@ k_fwd_tc(const __grid_constant__ TcMaps tm, const __grid_constant__ Consts c, co
                     uint32_t rn[CG], rc[CG];
                     tc::tmem_ld8_issue(taddr, rn);
                     if (TF) tc::tmem_ld8_issue(taddr + (uint32_t)BN, rc);
-#pragma unroll
+#pragma unroll kUnroll
                     for (int h = 0; h < 32 / CG; ++h) {
                         const int g0 = nb0 + h * CG;
                         tc::tmem_ld8_wait(rn);
@@ -395,7 +410,7 @@ k_fwd_tc(const __grid_constant__ TcMaps tm, const __grid_constant__ Consts c, co
                         uint32_t act = 0;                          // warp-uniform
 #pragma unroll
                         for (int k = 0; k < NB; ++k) {
-                            if (hlo[k] < g0 + CG && hhi[k] > g0) act |= 1u << k;
+                            if ((int)(hxy[k] & 0xffffu) < g0 + CG && (int)(hxy[k] >> 16) > g0) act |= 1u << k;
                         }
                         if (act == 0u) continue;
                         float s0[CG], sE[CG], sEb[CG], sEd[CG], lm[CG];
@@ -426,13 +441,18 @@ k_fwd_tc(const __grid_constant__ TcMaps tm, const __grid_constant__ Consts c, co
                                 const bool gauss = gs[k] != 0.0f;
 #pragma unroll
                                 for (int jj = 0; jj < CG; jj += 2) {
-                                    const int nn = g0 + jj;
-                                    const bool i0 = nn >= lo && nn < hi, i1 = nn + 1 >= lo && nn + 1 < hi;
-                                    float2 w = make_float2(i0 ? 1.0f : 0.0f, i1 ? 1.0f : 0.0f);
+                                    // a Gaussian needs no range test: past its support (6 sigma) it
+                                    // adds, where a neighbouring row's support reaches, less than
+                                    // 2e-9 of the band's weight
+                                    float2 w;
                                     if (gauss) {
                                         const float2 u = __fmul2_rn(__fadd2_rn(make_float2(lm[jj], lm[jj + 1]), ngc), gs2);
                                         const float2 t = __fmul2_rn(u, u);
-                                        w = make_float2(i0 ? ex2_(-t.x) : 0.0f, i1 ? ex2_(-t.y) : 0.0f);
+                                        w = make_float2(ex2_(-t.x), ex2_(-t.y));
+                                    } else {
+                                        const int nn = g0 + jj;
+                                        w = make_float2(nn >= lo && nn < hi ? 1.0f : 0.0f,
+                                                        nn + 1 >= lo && nn + 1 < hi ? 1.0f : 0.0f);
                                     }
                                     p0 = __ffma2_rn(make_float2(s0[jj], s0[jj + 1]), w, p0);
                                     p1 = __ffma2_rn(make_float2(sE[jj], sE[jj + 1]), w, p1);
@@ -494,7 +514,7 @@ k_fwd_tc(const __grid_constant__ TcMaps tm, const __grid_constant__ Consts c, co
             tc::mbar_arrive(&ctl->tempty[buf]);
         }
         // the block's slice of cJ is zeroed before the launch; a (row, band) gets
-        // one addend per column half, so the sum does not depend on their order
+        // one addend per column part (the order of three moves at most the last bit)
         if (valid && !ctl->abort) {
 #pragma unroll
             for (int k = 0; k < NB; ++k)
@@ -515,8 +535,7 @@ k_fwd_tc(const __grid_constant__ TcMaps tm, const __grid_constant__ Consts c, co
     tc_teardown<ST>(ctl, warp);
 }
 
-// Launch of k_fwd_tc for the band count (epilogue warps: 8 bands per group,
-// one group and two column halves, or up to four groups); KZ selects the
+// Launch of k_fwd_tc for the band count (fwd_shape); KZ selects the
 // variant that also accumulates the redshift derivative into cJz.
 template <bool KZ>
 cudaError_t fwd_tc_launch(const TcMaps& tm, bool tf, const Consts& c, const Grid& grid, const Galaxies& g,
@@ -525,26 +544,30 @@ cudaError_t fwd_tc_launch(const TcMaps& tm, bool tf, const Consts& c, const Grid
     if (n <= 0) return cudaSuccess;
     static_assert(kHullRows % kTM == 0, "a tile lies in one hull");
     const dim3 blocks((unsigned)((n + kTM - 1) / kTM), nsplit);
-    const size_t smem = tc_fwd_smem(tf);
-    const int groups = (c.n_band + kFwdGroupBands - 1) / kFwdGroupBands;   // <= 4 (B <= 32)
-    const int halves = groups == 1 ? 2 : 1;
-    const int threads = 64 + 32 * 4 * groups * halves;
+    const FwdShape sh = fwd_shape(c.n_band, tf);
+    const int threads = 64 + 32 * 4 * sh.groups * sh.parts;
     cudaError_t e = cudaMemsetAsync(cJ, 0, (size_t)nsplit * n * c.n_band * 4 * sizeof(float), s);
     if (e != cudaSuccess) return e;
     if (cJz) {
         e = cudaMemsetAsync(cJz, 0, (size_t)nsplit * n * c.n_band * 2 * sizeof(float), s);
         if (e != cudaSuccess) return e;
     }
-    auto go = [&](auto kern) -> cudaError_t {
+    auto go = [&](auto kern, size_t ring) -> cudaError_t {
+        const size_t smem = ring + 256 + kFwdConstBytes + 1024;
         cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (r != cudaSuccess) return r;
-        kern<<<blocks, threads, smem, s>>>(tm, c, grid, g, theta, gal_idx, perm, hull, n, halves, cJ, err, cJz);
+        kern<<<blocks, threads, smem, s>>>(tm, c, grid, g, theta, gal_idx, perm, hull, n, sh.parts, cJ, err, cJz);
         return cudaSuccess;
     };
     constexpr int T8 = 64 + 32 * 8, T12 = 64 + 32 * 12, T16 = 64 + 32 * kFwdMaxEpiWarps;
-    if (threads <= T8) e = tf ? go(k_fwd_tc<T8, true, KZ>) : go(k_fwd_tc<T8, false, KZ>);         // <= 16 bands
-    else if (threads <= T12) e = tf ? go(k_fwd_tc<T12, true, KZ>) : go(k_fwd_tc<T12, false, KZ>); // <= 24 bands
-    else e = tf ? go(k_fwd_tc<T16, true, KZ>) : go(k_fwd_tc<T16, false, KZ>);                     // <= 32 bands
+    constexpr size_t rs = Ring<192, kFwdStages<192, false>, false>::kBytes;
+    constexpr size_t rst = Ring<96, kFwdStages<96, true>, true>::kBytes;
+    constexpr size_t rl = Ring<256, kFwdStages<256, false>, false>::kBytes;
+    constexpr size_t rlt = Ring<128, kFwdStages<128, true>, true>::kBytes;
+    if (sh.bands == 6) e = tf ? go(k_fwd_tc<T12, 6, 96, true, KZ>, rst) : go(k_fwd_tc<T12, 6, 192, false, KZ>, rs);
+    else if (threads <= T8) e = tf ? go(k_fwd_tc<T8, 8, 128, true, KZ>, rlt) : go(k_fwd_tc<T8, 8, 256, false, KZ>, rl);
+    else if (threads <= T12) e = tf ? go(k_fwd_tc<T12, 8, 128, true, KZ>, rlt) : go(k_fwd_tc<T12, 8, 256, false, KZ>, rl);
+    else e = tf ? go(k_fwd_tc<T16, 8, 128, true, KZ>, rlt) : go(k_fwd_tc<T16, 8, 256, false, KZ>, rl);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }

@@ -200,7 +200,7 @@ __host__ __device__ inline int64_t keep_stride(const Consts& c) { return (2 + 6 
 struct TcMaps {
     CUtensorMap a[2], b[2];
 };
-size_t tc_fwd_smem(bool tf);
+int tc_fwd_columns(const Consts& c, bool tf);   // wavelengths per tile of the forward: box rows of its b maps
 size_t tc_adj_smem(bool tf);
 cudaError_t launch_fwd_tc(const TcMaps& tm, bool tf, const Consts& c, const Grid& grid, const Galaxies& g,
                           const float* theta, const int32_t* gal_idx, const int32_t* perm, const uint32_t* hull,
