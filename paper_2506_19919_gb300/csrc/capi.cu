@@ -740,8 +740,8 @@ sps_status sps_photometry(sps_ctx* ctx, const float* theta, const int32_t* gal_i
     if (sps_status r = st.check(); r != SPS_OK) return r;
     CK(cudaMemsetAsync(ctx->nonfinite.p, 0, 2 * sizeof(int), s));
     if (mode == SPS_APPROX && ctx->c.n_met <= 12 && !ctx->c.mdf_age && !std::getenv("SPS_LIKE_ROWS")) {
-        // forward-only team evaluation, one row per warp
-        CK(launch_phot_team(ctx->c, ctx->gal(), th, gi, n, mo, ctx->nonfinite.as<int>(), s));
+        // forward-only evaluation, one row per block (few rows) or per warp
+        CK((n <= approx_few_rows() ? launch_phot_few : launch_phot_team)(ctx->c, ctx->gal(), th, gi, n, mo, ctx->nonfinite.as<int>(), s));
     } else if (mode == SPS_APPROX) {
         CK(launch_approx_rows(ctx->c, ctx->gal(), th, 0, gi, n, nullptr, nullptr, nullptr, mo, nullptr,
                               nullptr, nullptr, ctx->nonfinite.as<int>(), s));
@@ -781,8 +781,8 @@ sps_status sps_loglike_grad(sps_ctx* ctx, const float* theta, const int32_t* gal
     if (sps_status r = st.check(); r != SPS_OK) return r;
     CK(cudaMemsetAsync(ctx->nonfinite.p, 0, 2 * sizeof(int), s));
     if (mode == SPS_APPROX && ctx->c.n_met <= 12 && !std::getenv("SPS_LIKE_ROWS")) {
-        // the team evaluation, one row per warp
-        CK(launch_like_team(ctx->c, ctx->gal(), th, gi, n, mo, sg, mk, llo, gro, ctx->nonfinite.as<int>(), s));
+        // one row per block (few rows of the separable model) or the team evaluation, one per warp
+        CK((n <= approx_few_rows() && !ctx->c.mdf_age ? launch_like_few : launch_like_team)(ctx->c, ctx->gal(), th, gi, n, mo, sg, mk, llo, gro, ctx->nonfinite.as<int>(), s));
     } else if (mode == SPS_APPROX) {
         CK(launch_approx_rows(ctx->c, ctx->gal(), th, 0, gi, n, mo, sg, mk, nullptr, llo, gro, nullptr,
                               ctx->nonfinite.as<int>(), s));

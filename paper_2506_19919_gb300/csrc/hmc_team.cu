@@ -81,11 +81,6 @@ __device__ __forceinline__ AgeView age_view(TeamWork<CPW>& t, int ch, const Edge
                    t.q[ch], t.qb[ch], &t.u.ps, et.age, et.lgz};
 }
 
-// Bring a band's c_SSP rows (n bytes, a multiple of 16 at a 16-byte boundary)
-// to L2 ahead of their use; one thread issues it.
-__device__ __forceinline__ void prefetch_l2(const float* p, uint32_t bytes) {
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
 constexpr int kAhead = 2;    // bands prefetched ahead
 
 // log posterior (unbounded space) and its gradient for every chain of the

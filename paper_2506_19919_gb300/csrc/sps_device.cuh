@@ -213,6 +213,12 @@ __device__ __forceinline__ void load_row(const float* __restrict__ p, int Zn, fl
     }
 }
 
+// Bring a band's c_SSP rows (n bytes, a multiple of 16 at a 16-byte boundary)
+// to L2 ahead of their use; one thread issues it.
+__device__ __forceinline__ void prefetch_l2(const float* p, uint32_t bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
 // ---------------------------------------------------------------- SFH bins
 // Panel count ceil(f) clamped to [1, kMaxPanels]; NaN or inf give a bounded
 // count so that no input can index outside the scratch arrays.
@@ -331,9 +337,11 @@ __device__ __forceinline__ void gl_panel_any(int n, const float* __restrict__ gx
 // ln tau + min(ln t_obs - ln tau, 0) - 22 / (beta + 1) the integrand is below
 // e^-22 of its value at the peak or at t_obs, and the remaining mass (< 1e-9
 // of the total) is dropped.
+// [i_begin, i_end): the bins to integrate (i_begin a multiple of 32; all by default).
 template <bool kPack = false>
 __device__ __forceinline__ void sfh_bins_raw(const Consts& c, const AgeView& v, const float2* __restrict__ bins,
-                                             float lnT, float tau, float alpha, float beta, bool grad) {
+                                             float lnT, float tau, float alpha, float beta, bool grad,
+                                             int i_begin = 0, int i_end = kMaxAges) {
     PanelScratch& ps = *v.ps;
     const int lane = lane_id();
     const int A = c.n_age;
@@ -349,7 +357,7 @@ __device__ __forceinline__ void sfh_bins_raw(const Consts& c, const AgeView& v, 
     // integrated here, a bin of several panels is queued for pass 2.
     int base = 0;                               // panels queued so far (warp-uniform)
 #pragma unroll 1
-    for (int i0 = 0; i0 < A; i0 += 32) {
+    for (int i0 = i_begin; i0 < A && i0 < i_end; i0 += 32) {
         const int i = i0 + lane;
         int n = 0;
         float x0 = 0.0f, hp = 0.0f;
