@@ -36,15 +36,34 @@ def _stream(t):
     return None
 
 
+def _ready(x, dtype, device=None):
+    """Whether x can be handed to the library as it is: a plain contiguous
+    tensor of that type on that device (conversions that change nothing still
+    cost a call to the dispatcher each, about 20 us for the arguments of one call)."""
+    return (isinstance(x, torch.Tensor) and x.dtype is dtype and (device is None or x.device == device)
+            and x.is_contiguous())
+
+
+def _i32(x, device):
+    """Galaxy indices as a contiguous int32 tensor on `device`."""
+    if x is None or _ready(x, torch.int32, device):
+        return x
+    return torch.as_tensor(x, dtype=torch.int32, device=device).contiguous()
+
+
 def _f32(x, device=None):
     """x as a contiguous float32 tensor on `device` (a tensor's own device when
     None); a tensor that already is one is returned as it is, without a copy."""
+    if _ready(x, torch.float32, device):
+        return x
     t = torch.as_tensor(x)
     return t.to(device=t.device if device is None else device, dtype=torch.float32).contiguous()
 
 
 def _mask32(mask, device):
     """Band bitmasks as a contiguous int32 tensor holding the uint32 bits."""
+    if _ready(mask, torch.int32, device):
+        return mask
     if isinstance(mask, torch.Tensor):
         if mask.dtype != torch.int32:
             mask = torch.as_tensor(np.asarray(mask.cpu().numpy(), dtype=np.int64).astype(np.uint32).view(np.int32))
@@ -148,8 +167,7 @@ class Context:
         n = th.shape[0]
         if out is None:
             out = torch.empty((n, self.n_band), dtype=torch.float32, device=th.device)
-        gi = None if gal_idx is None else torch.as_tensor(gal_idx, dtype=torch.int32,
-                                                             device=th.device).contiguous()
+        gi = _i32(gal_idx, th.device)
         check(self._lib.sps_photometry(self.h, _vp(th), _vp(gi), n, MODES[mode], PRECS[prec],
                                        _vp(out), _stream(th)), "sps_photometry")
         return out
@@ -162,8 +180,7 @@ class Context:
         mo = _f32(mag_obs, dev)
         sg = _f32(sigma, dev)
         mk = _mask32(mask, dev)
-        gi = None if gal_idx is None else torch.as_tensor(gal_idx, dtype=torch.int32,
-                                                             device=dev).contiguous()
+        gi = _i32(gal_idx, dev)
         ll = torch.empty(n, dtype=torch.float32, device=dev)
         g = torch.empty((n, _lib.NPARAM), dtype=torch.float32, device=dev) if grad else None
         check(self._lib.sps_loglike_grad(self.h, _vp(th), _vp(gi), n, _vp(mo), _vp(sg), _vp(mk),
@@ -180,8 +197,7 @@ class Context:
         mo = _f32(mag_obs, dev)
         sg = _f32(sigma, dev)
         mk = _mask32(mask, dev)
-        gi = None if gal_idx is None else torch.as_tensor(gal_idx, dtype=torch.int32,
-                                                             device=dev).contiguous()
+        gi = _i32(gal_idx, dev)
         ll = torch.empty(n, dtype=torch.float32, device=dev)
         g = torch.empty((n, _lib.NPARAM + 1), dtype=torch.float32, device=dev)
         check(self._lib.sps_loglike_grad_z(self.h, _vp(th), _vp(gi), n, _vp(mo), _vp(sg), _vp(mk),
@@ -197,8 +213,7 @@ class Context:
         mo = _f32(mag_obs, dev)
         sg = _f32(sigma, dev)
         mk = _mask32(mask, dev)
-        gi = None if gal_idx is None else torch.as_tensor(gal_idx, dtype=torch.int32,
-                                                             device=dev).contiguous()
+        gi = _i32(gal_idx, dev)
         ll = torch.empty(n, dtype=torch.float32, device=dev)
         g = torch.empty((n, _lib.NPARAM), dtype=torch.float32, device=dev)
         check(self._lib.sps_loglike_grad_forward_mode(self.h, _vp(th), _vp(gi), n, _vp(mo), _vp(sg),
@@ -258,8 +273,7 @@ class Context:
         l = torch.as_tensor(L, dtype=torch.int32).to(dev).contiguous()
         mo, sg = _f32(mag_obs, dev), _f32(sigma, dev)
         mk = torch.as_tensor(np.asarray(mask, dtype=np.uint32).view(np.int32)).to(dev).contiguous()
-        gi = None if gal_idx is None else torch.as_tensor(gal_idx, dtype=torch.int32,
-                                                             device=dev).contiguous()
+        gi = _i32(gal_idx, dev)
         xo = torch.empty_like(x)
         po = torch.empty_like(x)
         lo = torch.empty(n, dtype=torch.float64, device=dev)
@@ -287,8 +301,7 @@ class Context:
         info = self.info()
         W = torch.empty((n, info["n_age"] * info["n_met"]), dtype=torch.float32, device=th.device)
         M = torch.empty(n, dtype=torch.float64, device=th.device)
-        gi = None if gal_idx is None else torch.as_tensor(gal_idx, dtype=torch.int32,
-                                                             device=th.device).contiguous()
+        gi = _i32(gal_idx, th.device)
         check(self._lib.sps_weights(self.h, _vp(th), _vp(gi), n, _vp(W), _vp(M), _stream(th)),
               "sps_weights")
         return W, M

@@ -83,6 +83,7 @@ struct sps_ctx {
     DevBuf cJz, rowz;                 // exact path: the z accumulators and explicit z term
     // scratch
     DevBuf nonfinite, queue, err;
+    int* flags = nullptr;             // pinned copy of the nonfinite / error words
     DevBuf W, V, Wbar, cJ, gbar, rowinfo, tcerr, plainT, plainC, hmcm;
     DevBuf pst, pth, pll, pgr, pgi;   // plain lock-step HMC state and gradient buffers
     DevBuf hmcn;                      // NUTS tree state per chain
@@ -141,6 +142,7 @@ struct sps_ctx {
         if (fork) cudaEventDestroy(fork);
         if (join) cudaEventDestroy(join);
         if (side) cudaStreamDestroy(side);
+        if (flags) cudaFreeHost(flags);
         DevBuf* all[] = {&lam64, &lam32, &lamc, &lamq, &lamd, &lamdq, &gl32, &prep, &ssp, &ssp_t, &ssp_bf, &ssp_t_bf, &row_scale, &col_scale,
                          &age_edges, &bp0, &bp1, &gz, &glnT, &glT10, &gbins, &gzp, &gsup, &ggauss,
                          &gcssp, &gdust, &gdtdz, &gdzp, &gddust, &gdcssp, &cJz, &rowz, &nonfinite, &queue, &err, &W, &V, &Wbar, &cJ, &gbar,
