@@ -504,7 +504,7 @@ sps_status sps_create(sps_ctx** out, const sps_tables* t, const sps_config* cfg_
         (e = upload(ctx->gl32, gl32, sizeof(gl32))) != cudaSuccess ||
         (e = ctx->lam32.reserve(sizeof(float) * L)) != cudaSuccess ||
         (e = ctx->lamc.reserve(sizeof(float4) * L)) != cudaSuccess ||
-        (e = ctx->lamq.reserve(sizeof(float2) * L)) != cudaSuccess ||
+        (e = ctx->lamp.reserve(sizeof(float) * 6 * (size_t)lp)) != cudaSuccess ||
         (e = ctx->lamd.reserve(sizeof(float4) * L)) != cudaSuccess ||
         (e = ctx->lamdq.reserve(sizeof(float2) * L)) != cudaSuccess ||
         (e = ctx->nonfinite.reserve(64)) != cudaSuccess || (e = ctx->queue.reserve(64)) != cudaSuccess ||
@@ -514,9 +514,9 @@ sps_status sps_create(sps_ctx** out, const sps_tables* t, const sps_config* cfg_
         return (e == cudaErrorMemoryAllocation) ? fail(SPS_E_NOMEM, "table upload: out of memory")
                                                 : cuda_fail(e, "table upload");
     }
-    if ((e = launch_lambda_consts(ctx->lam64.as<double>(), L, ctx->lamc.as<float4>(),
-                                  ctx->lam32.as<float>(), ctx->lamq.as<float2>(), ctx->lamd.as<float4>(),
-                                  ctx->lamdq.as<float2>(), 0)) != cudaSuccess ||
+    if ((e = launch_lambda_consts(ctx->lam64.as<double>(), L, lp, ctx->lamc.as<float4>(), ctx->lam32.as<float>(),
+                                  ctx->lamd.as<float4>(), ctx->lamdq.as<float2>(), ctx->lamp.as<float>(), 0)) !=
+            cudaSuccess ||
         (e = cudaDeviceSynchronize()) != cudaSuccess) {
         delete ctx;
         return cuda_fail(e, "lambda constants");

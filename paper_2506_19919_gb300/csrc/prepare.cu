@@ -52,12 +52,19 @@ __device__ double drude_dshape(double lum) {
 }
 
 // Per-wavelength constants: (q_n / lambda_n, k0, ln(lambda/lambda_V), Drude),
-// and lambda, q / lambda, q as double-float pairs for the set-up kernels.
-__global__ void k_lambda_consts(const double* __restrict__ lam, int L, float4* __restrict__ out,
-                                float* __restrict__ lam32, float2* __restrict__ lamq,
-                                float4* __restrict__ lamd, float2* __restrict__ lamdq) {
+// lambda, q / lambda, q as double-float pairs for the set-up kernels, and the
+// constants of neighbouring wavelengths side by side for packed arithmetic
+// (lamp; zero past the grid).
+__global__ void k_lambda_consts(const double* __restrict__ lam, int L, int lam_pad, float4* __restrict__ out,
+                                float* __restrict__ lam32, float4* __restrict__ lamd, float2* __restrict__ lamdq,
+                                float* __restrict__ lamp) {
     int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= L) return;
+    if (n >= lam_pad) return;
+    float* pr = lamp + 12 * (n >> 1) + (n & 1);
+    if (n >= L) {
+        for (int k = 0; k < 12; k += 2) pr[k] = 0.0f;
+        return;
+    }
     double l = lam[n];
     double q = (n == 0) ? 0.5 * (lam[1] - lam[0])
              : (n == L - 1) ? 0.5 * (lam[L - 1] - lam[L - 2])
@@ -66,7 +73,12 @@ __global__ void k_lambda_consts(const double* __restrict__ lam, int L, float4* _
     out[n] = make_float4((float)(q / l), (float)calzetti_k0(lum), (float)log(l / 5500.0),
                          (float)drude_shape(lum));
     lam32[n] = (float)l;
-    lamq[n] = make_float2((float)l, (float)(q / l));
+    pr[0] = (float)l;
+    pr[2] = (float)(q / l);
+    pr[4] = out[n].y;
+    pr[6] = out[n].z;
+    pr[8] = out[n].w;
+    pr[10] = 0.0f;
     const Df ld = df_from(l), rd = df_from(q / l), qd = df_from(q);
     lamd[n] = make_float4(ld.h, ld.l, rd.h, rd.l);
     lamdq[n] = make_float2(qd.h, qd.l);
@@ -460,9 +472,9 @@ k_cssp(const __grid_constant__ Consts c, const Grid grid, const Galaxies gal, co
 
 }  // namespace
 
-cudaError_t launch_lambda_consts(const double* lam, int L, float4* out, float* lam32, float2* lamq, float4* lamd,
-                                 float2* lamdq, cudaStream_t s) {
-    k_lambda_consts<<<(L + 255) / 256, 256, 0, s>>>(lam, L, out, lam32, lamq, lamd, lamdq);
+cudaError_t launch_lambda_consts(const double* lam, int L, int lam_pad, float4* out, float* lam32, float4* lamd,
+                                 float2* lamdq, float* lamp, cudaStream_t s) {
+    k_lambda_consts<<<(lam_pad + 255) / 256, 256, 0, s>>>(lam, L, lam_pad, out, lam32, lamd, lamdq, lamp);
     return cudaGetLastError();
 }
 

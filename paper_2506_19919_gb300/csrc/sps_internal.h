@@ -63,7 +63,8 @@ struct Galaxies {
 struct Grid {
     const float* lam;        // [L] Angstrom
     const float4* lamc;      // [L] (q_n / lambda_n, k0, ln(lambda/lambda_V), Drude shape)
-    const float2* lamq;      // [L] (lambda, q_n / lambda_n) in FP32
+    const float4* lamp;      // [lam_pad / 2][3] wavelength pairs: (lambda, lambda', q / lambda, q' / lambda'),
+                             // (k0, k0', ln(l / l_V), ln(l' / l_V)), (Drude, Drude', 0, 0)
     const double* lam64;     // [L] Angstrom, FP64
     const float4* lamd;      // [L] lambda and q_n / lambda_n as double-float pairs (hi, lo, hi, lo)
     const float2* lamdq;     // [L] q_n as a double-float pair
@@ -162,8 +163,8 @@ cudaError_t launch_exact_fwd(const Consts& c, const Grid& grid, const Galaxies& 
                              const int32_t* gal_idx, const int32_t* perm, int64_t n, int bf16, const float* W32,
                              const uint16_t* Wbf, float* cJ, int nsplit, cudaStream_t s,
                              float* cJz = nullptr);   // with cJz: [r][b][2] sum_n wb' S (1, E)
-cudaError_t launch_lambda_consts(const double* lam, int L, float4* out, float* lam32, float2* lamq, float4* lamd,
-                                 float2* lamdq, cudaStream_t s);
+cudaError_t launch_lambda_consts(const double* lam, int L, int lam_pad, float4* out, float* lam32, float4* lamd,
+                                 float2* lamdq, float* lamp, cudaStream_t s);
 cudaError_t launch_exact_like(const Consts& c, const Galaxies& g, const float* theta,
                               const int32_t* gal_idx, int64_t n, const float* cJ, float* rowinfo,
                               const float* mag_obs, const float* sigma, const uint32_t* mask,
