@@ -1,6 +1,8 @@
 // Approximate photometry, log-likelihood and adjoint gradient, one warp per
 // row (Eq. photo_integral_approx, App. D.1), plus the SSP-weights and Philox
 // test hooks.
+#include <algorithm>
+
 #include "sps_eval.cuh"
 #include "philox.cuh"
 
@@ -8,23 +10,38 @@ namespace sps {
 
 namespace {
 
-__global__ void __launch_bounds__(32 * kWarpsApprox)
+// One row per warp; the warps of a block meet once per row, which keeps their
+// code in the instruction cache.  Bound by the latency of the c_SSP rows (5 KB
+// per band and warp): they are loaded without a predicate per column and come
+// to L2 two bands early.  With the redshift column six warps of 168 registers,
+// two blocks per SM: 25,000 rows of six bands 0.60 ms a call (2.16 ms with four
+// warps, no barrier and predicated loads at 128 registers; twelve, ten or eight
+// warps in one block 0.63, 0.69, 0.71; eight warps of 128 registers spill, 1.56).
+// Without it eight warps of 128: photometry of 30,000 rows with an age-dependent
+// MDF 0.45 ms (0.70 before; six warps 0.53).
+constexpr int kWarpsRow = 8;
+constexpr int kWarpsRowZ = 6;
+
+__global__ void __launch_bounds__(32 * kWarpsRow, 2)
 k_approx_rows(const __grid_constant__ Consts c, const Galaxies g, const float* __restrict__ theta,
               int unbounded, const int32_t* __restrict__ gal_idx, int64_t n,
               const float* __restrict__ mag_obs, const float* __restrict__ sigma,
               const uint32_t* __restrict__ mask, float* __restrict__ mag_out,
               float* __restrict__ ll_out, float* __restrict__ grad_out,
               double* __restrict__ logp_out, int* __restrict__ nonfinite) {
-    __shared__ WarpWork work[kWarpsApprox];
-    const int warp = threadIdx.x >> 5;
+    extern __shared__ __align__(16) unsigned char smem[];
+    WarpWork* work = reinterpret_cast<WarpWork*>(smem);
+    const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5;
     const int lane = lane_id();
     WarpWork& ww = work[warp];
     const bool like = (ll_out != nullptr) || (logp_out != nullptr);
     const bool grad = grad_out != nullptr;
     const int B = c.n_band;
     const uint32_t all = (B >= 32) ? 0xffffffffu : ((1u << B) - 1u);
-    for (int64_t row = (int64_t)blockIdx.x * kWarpsApprox + warp; row < n;
-         row += (int64_t)gridDim.x * kWarpsApprox) {
+    for (int64_t base = (int64_t)blockIdx.x * warps; base < n; base += (int64_t)gridDim.x * warps) {
+        __syncthreads();
+        const int64_t row = base + warp;
+        if (row >= n) continue;
         const int64_t gi = gal_idx ? (int64_t)gal_idx[row] : row;
         RowParams p;
         load_params(c, theta + row * SPS_NPARAM, unbounded != 0, p);
@@ -65,20 +82,23 @@ k_approx_rows(const __grid_constant__ Consts c, const Galaxies g, const float* _
 
 // log L and d log L / d(theta, z) of the approximate path, one warp per row:
 // grad_out[row][13], the last column the derivative in the galaxy's redshift.
-__global__ void __launch_bounds__(32 * kWarpsApprox)
+__global__ void __launch_bounds__(32 * kWarpsRowZ, 2)
 k_approx_rows_z(const __grid_constant__ Consts c, const Galaxies g, const float* __restrict__ theta,
                 const int32_t* __restrict__ gal_idx, int64_t n, const float* __restrict__ mag_obs,
                 const float* __restrict__ sigma, const uint32_t* __restrict__ mask,
                 float* __restrict__ ll_out, float* __restrict__ grad_out, int* __restrict__ nonfinite) {
-    __shared__ WarpWork work[kWarpsApprox];
-    const int warp = threadIdx.x >> 5;
+    extern __shared__ __align__(16) unsigned char smem[];
+    WarpWork* work = reinterpret_cast<WarpWork*>(smem);
+    const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5;
     const int lane = lane_id();
     WarpWork& ww = work[warp];
     const int B = c.n_band;
     constexpr int NG = SPS_NPARAM + 1;
     const uint32_t all = (B >= 32) ? 0xffffffffu : ((1u << B) - 1u);
-    for (int64_t row = (int64_t)blockIdx.x * kWarpsApprox + warp; row < n;
-         row += (int64_t)gridDim.x * kWarpsApprox) {
+    for (int64_t base = (int64_t)blockIdx.x * warps; base < n; base += (int64_t)gridDim.x * warps) {
+        __syncthreads();
+        const int64_t row = base + warp;
+        if (row >= n) continue;
         const int64_t gi = gal_idx ? (int64_t)gal_idx[row] : row;
         RowParams p;
         load_params(c, theta + row * SPS_NPARAM, false, p);
@@ -158,6 +178,9 @@ int blocks_for(int64_t rows, int per_block) {
     if (b > 152LL * 64) b = 152LL * 64;
     return (int)(b < 1 ? 1 : b);
 }
+// Fewer rows than fill every SM's block take one warp per block and SM, then two,
+// and so on: 50 rows with the redshift column 67 us a call, 133 us before, four a block.
+int row_warps(int64_t n, int most) { return (int)std::min<int64_t>(most, (n + kSms - 1) / kSms); }
 
 }  // namespace
 
@@ -167,7 +190,11 @@ cudaError_t launch_approx_rows(const Consts& c, const Galaxies& g, const float* 
                                float* mag_out, float* loglike_out, float* grad_out,
                                double* logp_out, int* nonfinite, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    k_approx_rows<<<blocks_for(n, kWarpsApprox), 32 * kWarpsApprox, 0, s>>>(
+    const int warps = row_warps(n, kWarpsRow);
+    cudaError_t e = cudaFuncSetAttribute(k_approx_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(kWarpsRow * sizeof(WarpWork)));
+    if (e != cudaSuccess) return e;
+    k_approx_rows<<<blocks_for(n, warps), 32 * warps, warps * sizeof(WarpWork), s>>>(
         c, g, theta, theta_unbounded, gal_idx, n, mag_obs, sigma, mask, mag_out, loglike_out,
         grad_out, logp_out, nonfinite);
     return cudaGetLastError();
@@ -178,7 +205,11 @@ cudaError_t launch_approx_rows_z(const Consts& c, const Galaxies& g, const float
                                  const float* sigma, const uint32_t* mask, float* loglike_out,
                                  float* grad_out, int* nonfinite, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
-    k_approx_rows_z<<<blocks_for(n, kWarpsApprox), 32 * kWarpsApprox, 0, s>>>(
+    const int warps = row_warps(n, kWarpsRowZ);
+    cudaError_t e = cudaFuncSetAttribute(k_approx_rows_z, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)(kWarpsRowZ * sizeof(WarpWork)));
+    if (e != cudaSuccess) return e;
+    k_approx_rows_z<<<blocks_for(n, warps), 32 * warps, warps * sizeof(WarpWork), s>>>(
         c, g, theta, gal_idx, n, mag_obs, sigma, mask, loglike_out, grad_out, nonfinite);
     return cudaGetLastError();
 }

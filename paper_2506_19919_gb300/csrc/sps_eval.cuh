@@ -77,20 +77,39 @@ __device__ inline double eval_row(const Consts& c, WarpWork& ww, const float2* _
     // with an age-dependent MDF, w_i q_ij with q_ij staged in kbuf
     const bool nonsep = c.mdf_age != 0;
     if (nonsep) mdf_rows_fill(c, c.lgz_edge, p.th[7], p.th[8], s.u.kbuf);
+    // ((age, metallicity) of a column is stepped along, not divided out)
     float wreg[kKTileMax];
+    const int di = 32 / Zn, dj = 32 % Zn;
+    int ki = lane / Zn, kj = lane % Zn;
 #pragma unroll
     for (int t = 0; t < kKTileMax; ++t) {
         int k = lane + 32 * t;
-        wreg[t] = (k < K) ? s.w[k / Zn] * (nonsep ? s.u.kbuf[k] : s.q[k % Zn]) : 0.0f;
+        wreg[t] = (k < K) ? s.w[ki] * (nonsep ? s.u.kbuf[k] : s.q[kj]) : 0.0f;
+        ki += di;
+        kj += dj;
+        if (kj >= Zn) {
+            kj -= Zn;
+            ++ki;
+        }
     }
     __syncwarp();
+    const bool ahead = (K & 3) == 0;           // the bands' rows to L2 two bands early
+    if (ahead && lane < min(2, nb)) {
+        prefetch_l2(d.ptr[lane], 4u * K);
+        if (kZ) prefetch_l2(zr->dcssp + (size_t)d.band[lane] * K, 4u * K);
+    }
     for (int sl = 0; sl < nb; ++sl) {
         const float* C = d.ptr[sl];
+        if (ahead && lane == 0 && sl + 2 < nb) {
+            prefetch_l2(d.ptr[sl + 2], 4u * K);
+            if (kZ) prefetch_l2(zr->dcssp + (size_t)d.band[sl + 2] * K, 4u * K);
+        }
+        // columns past the table have weight 0 and read its last one: without a
+        // predicate per column the loads of a row are in flight together
         float a = 0.0f;
 #pragma unroll
         for (int t = 0; t < kKTileMax; ++t) {
-            int k = lane + 32 * t;
-            if (k < K) a = fmaf(wreg[t], C[k], a);
+            a = fmaf(wreg[t], C[min(lane + 32 * t, K - 1)], a);
         }
         a = warp_sum(a);
         if (lane == 0) s.slot_S[sl] = a;
@@ -99,8 +118,7 @@ __device__ inline double eval_row(const Consts& c, WarpWork& ww, const float2* _
             float b = 0.0f;
 #pragma unroll
             for (int t = 0; t < kKTileMax; ++t) {
-                int k = lane + 32 * t;
-                if (k < K) b = fmaf(wreg[t], Cd[k], b);
+                b = fmaf(wreg[t], Cd[min(lane + 32 * t, K - 1)], b);
             }
             b = warp_sum(b);
             if (lane == 0) s.slot_D[sl] = b;
@@ -155,15 +173,22 @@ __device__ inline double eval_row(const Consts& c, WarpWork& ww, const float2* _
     gdl = warp_sum(gdl);
     gff = warp_sum(gff);
     __syncwarp();
-    // v_k = sum_b (gamma_b / S_b) c_SSP[b][k]
-#pragma unroll 4
+    // v_k = sum_b (gamma_b / S_b) c_SSP[b][k], band by band, a row's loads together
+    float v[kKTileMax];
+#pragma unroll
+    for (int t = 0; t < kKTileMax; ++t) v[t] = 0.0f;
+    for (int sl = 0; sl < nb; ++sl) {
+        const float* C = d.ptr[sl];
+        const float gb = s.slot_g[sl];
+#pragma unroll
+        for (int t = 0; t < kKTileMax; ++t) {
+            v[t] = fmaf(gb, C[min(lane + 32 * t, K - 1)], v[t]);
+        }
+    }
+#pragma unroll
     for (int t = 0; t < kKTileMax; ++t) {
         int k = lane + 32 * t;
-        if (k < K) {
-            float v = 0.0f;
-            for (int sl = 0; sl < nb; ++sl) v = fmaf(s.slot_g[sl], d.ptr[sl][k], v);
-            s.u.kbuf[k] = v;
-        }
+        if (k < K) s.u.kbuf[k] = v[t];
     }
     __syncwarp();
     float g[SPS_NPARAM];
@@ -182,11 +207,15 @@ __device__ inline double eval_row(const Consts& c, WarpWork& ww, const float2* _
             for (int j = 0; j < Zn; ++j) a = fmaf(vr[j], s.q[j], a);
             s.wb[i] = a;
         }
-        if (lane < Zn) {
-            float a = 0.0f;
-            for (int i = 0; i < A; ++i) a = fmaf(s.u.kbuf[i * Zn + lane], s.w[i], a);
-            s.qb[lane] = a;
+        // qbar_j = sum_i w_i v_ij: the lanes take (part of the ages, j)
+        const int parts = max(1, 32 / Zn), part = lane / Zn, j = lane - part * Zn;
+        float a = 0.0f;
+        if (part < parts) {
+            for (int i = part; i < A; i += parts) a = fmaf(s.u.kbuf[i * Zn + j], s.w[i], a);
         }
+        float qsum = a;
+        for (int o = 1; o < parts; ++o) qsum += __shfl_sync(0xffffffffu, a, (lane + o * Zn) & 31);
+        if (lane < Zn) s.qb[lane] = qsum;
         __syncwarp();
     }
     age_met_adjoint(c, s, lT10, M, p, g);
