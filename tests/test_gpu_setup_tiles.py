@@ -30,7 +30,7 @@ def _tables(tophat):
     return W.with_bands(base, kind, p0, p1, tn.astype(np.int32), tT)
 
 
-@pytest.mark.parametrize("n", [1, 3, 4, 5, 17, 511, 512, 529])
+@pytest.mark.parametrize("n", [1, 3, 4, 5, 17, 319, 320, 511, 512, 529])
 def test_setup_tiles_match_oracle(n):
     import paper_2506_19919_gb300 as pkg
     rng = np.random.default_rng(100 + n)
