@@ -183,7 +183,7 @@ sps_status sps_create(sps_ctx** out, const sps_tables* tables, const sps_config*
 sps_status sps_destroy(sps_ctx* ctx);
 
 /* Set the galaxies (their redshifts z[n_gal], float32) that later rows refer to.
- * Computes per galaxy, in FP64: t_obs(z), d_L(z), the age bins in cosmic time
+ * Computes per galaxy, in FP64 and (the wavelength sums) double-float: t_obs(z), d_L(z), the age bins in cosmic time
  * (Eq. smoothPsfh), band supports, band normalisations and AB zero points, and,
  * if build_approx != 0, lambda_eff (Eq. lambda_eff) and the per-galaxy table
  * c_SSP[g][b][ij] (the c_SSP definition of Sec. 3, "at a fixed z if the

@@ -67,7 +67,7 @@ k_adj_tc(const __grid_constant__ TcMaps tm, const __grid_constant__ Consts c, co
 
     // v is zero outside the hull of the rows' supports: the reduction covers its
     // k-blocks only (the grid's last one reads zero fill); 100,000 rows, six bands:
-    // 0.64 ms against 1.11 ms over the whole grid
+    // 0.64 ms against 1.11 ms over the whole grid (both before the stores below)
     const int2 hr = row_hull(c, hull, m0);
     // and of these the block takes part blockIdx.y of gridDim.y, into its own
     // slice of Wbar
