@@ -48,6 +48,7 @@ ESS_TARGET = 100.0
 # 0.72 -> 4,689, 0.75 -> 4,627, 0.8 (the library default) -> 4,286, 0.9 -> 3,179.
 TARGET_ACCEPT = 0.7
 METRIC = "posteriors/min at fixed ESS"
+GAUSS_SIGMA_PER_FWHM = 0.42466090014400953      # 1 / (2 sqrt(2 ln 2))
 UNIT = "posteriors/min"
 
 # DRAM traffic of one bench step's k_hmc_team launches on this workload (the
@@ -178,6 +179,17 @@ def _hmc_workload(rank: int, n_gal: int | None = None, iters=None):
     if iters is not None:                      # reduced run for profiling captures only
         wl.extra["n_warm"], wl.extra["n_samp"] = iters
     return wl
+
+
+def _lam_in_supports(wl):
+    """Grid wavelengths inside at least one (Gaussian, 6 sigma) band support,
+    averaged over the galaxies' redshifts (quantiles)."""
+    t = wl.tables
+    half = 6.0 * np.asarray(t.band_p1) * GAUSS_SIGMA_PER_FWHM
+    lo, hi = np.asarray(t.band_p0) - half, np.asarray(t.band_p0) + half
+    zs = np.quantile(np.asarray(wl.z), np.linspace(0.005, 0.995, 100))
+    x = (1.0 + zs)[:, None, None] * np.asarray(t.lam_ang)
+    return float(((x > lo[:, None]) & (x < hi[:, None])).any(1).sum(1).mean())
 
 
 def _config(tables, G, C, n_warm, n_samp, L, sampler, mdf_age, ws):
@@ -660,13 +672,14 @@ def _loglike_grad_rates(ctx_hmc, dev):
         torch.cuda.synchronize()
         return e0.elapsed_time(e1) / reps
 
-    # tensor-core throughput of the exact path: 2 K Lambda FLOP per row and
-    # contraction (the unpadded grid), one contraction for photometry and two
+    # tensor-core throughput of the exact path: 2 K FLOP per row, contraction and
+    # grid wavelength inside one of the row's band supports (the others have no
+    # weight and are not computed), one contraction for photometry and two
     # (forward and adjoint) for log L + gradient; BF16 against the measured
     # BF16 peak, 3xTF32 (three TF32 products per FLOP) against that peak times
     # the nominal TF32 / BF16 ratio 1.1 / 2.25
     peaks, src = _peaks()
-    flop_row = 2.0 * wl.tables.n_age * wl.tables.n_met * wl.tables.n_lam
+    flop_row = 2.0 * wl.tables.n_age * wl.tables.n_met * _lam_in_supports(wl)
 
     def tensor(ms, n_gemm, prec):
         if prec not in ("bf16", "tf32x3"):
