@@ -440,8 +440,8 @@ __device__ __forceinline__ void sfh_bins_raw(const Consts& c, const AgeView& v, 
         // flag = bin index at a bin's first panel; the running max gives the bin
         int f = -1;
         if (act) {
-            const int cand = ps.pmap[p];
-            if (cand < A && __float_as_int(ps.info[cand].z) == p) f = cand;
+            const int cand = ps.pmap[p];        // may be left from an earlier call, as is info outside the range
+            if (cand >= i_begin && cand < min(i_end, A) && __float_as_int(ps.info[cand].z) == p) f = cand;
         }
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {

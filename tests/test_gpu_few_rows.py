@@ -72,3 +72,32 @@ def test_few_rows_match_general_path_and_oracle(n_age, n_met, n_band, n):
     out = out.cpu().numpy()
     assert np.isnan(out[0]).all() and (n == 1 or np.array_equal(out[1:], m[1:]))
     ctx.close()
+
+
+@pytest.mark.parametrize("n_age,n_met", [(33, 10), (70, 12), (107, 12)])
+def test_few_rows_after_other_kernels(n_age, n_met):
+    """The block-per-row kernel reads no quadrature bookkeeping that another
+    kernel left in shared memory: log L + gradient of the same rows before and
+    after calls that integrate other rows with other layouts."""
+    import paper_2506_19919_gb300 as pkg
+    rng = np.random.default_rng(n_age)
+    tabs = W.make_tables(rng, n_age, n_met, 401, 900.0, 12000.0, W._gauss_bands([3600.0, 5200.0, 7600.0]))
+    G, n = 9, 760
+    z = rng.uniform(0.05, 1.0, G).astype(np.float32).astype(np.float64)
+    idx = rng.integers(0, G, n).astype(np.int32)
+    th = W.prior_draw(rng, n)
+    ctx = pkg.Context(tabs)
+    ctx.set_galaxies(z, build_approx=True)
+    obs, sigma, mask = np.full((G, 3), 15.0), np.full((G, 3), 0.05), np.full(G, 7, np.uint32)
+    call = lambda: [x.cpu().numpy() for x in ctx.loglike_grad(th, obs, sigma, mask, gal_idx=idx)]   # noqa: E731
+    ll, g = _general(call)
+    other = W.prior_draw(rng, 2000)
+    oi = rng.integers(0, G, 2000).astype(np.int32)
+    for mode in ("exact", "approx"):
+        for _ in range(3):
+            ctx.photometry(other, gal_idx=oi, mode=mode)
+            ctx.loglike_grad(other, obs, sigma, mask, gal_idx=oi, mode=mode)
+            l1, g1 = call()
+            assert (np.abs(g1 - g).max(1) / np.abs(g).max(1)).max() < 1e-4
+            np.testing.assert_allclose(l1, ll, rtol=1e-5)
+    ctx.close()
