@@ -7,14 +7,11 @@
 // sums over ages and bands meet in shared memory.
 // A call on 64 rows of six bands takes 55.5 us against 63 (photometry 45 against
 // 47), most of the rest in the host's part.
-#include "sps_device.cuh"
+#include "few.cuh"
 
 namespace sps {
 
 namespace {
-
-constexpr int kFewWarps = 4, kFewThreads = 32 * kFewWarps;
-static_assert(kFewThreads == kMaxAges, "one thread per age bin");
 
 struct FewWork {
     float m[kMaxAges], dm0[kMaxAges], dm1[kMaxAges], dm2[kMaxAges], pi[kMaxAges], w[kMaxAges], wb[kMaxAges];
@@ -239,56 +236,13 @@ k_approx_few(const __grid_constant__ Consts c, const Galaxies g, const float* __
         }
     }
     __syncthreads();
-    // ---- through the SFH, burst and MDF weights (the sums of age_met_adjoint)
-    float a[SPS_NPARAM];
-    {
-        const float w0 = t < A ? wb : 0.0f;
-        const float d0 = t < A ? s.dm0[t] : 0.0f, d1 = t < A ? s.dm1[t] : 0.0f, d2 = t < A ? s.dm2[t] : 0.0f;
-        a[0] = w0 * pi;
-        a[1] = w0 * mi;
-        a[2] = w0 * d0;
-        a[3] = w0 * d1;
-        a[4] = w0 * d2;
-        a[5] = d0;
-        a[6] = d1;
-        a[7] = d2;
-        a[8] = a[9] = a[10] = a[11] = 0.0f;
-        // burst, edge by edge
-        for (int e = t; e <= A; e += kFewThreads) {
-            const float x = (fminf(et.age[e], lT10) - mu) * isig;
-            const float dd = ((e < A) ? s.wb[e] : 0.0f) - ((e > 0) ? s.wb[e - 1] : 0.0f);
-            const float tp = tri_pdf(x) * dd;
-            a[8] += tp;
-            a[9] = fmaf(x, tp, a[9]);
-        }
-        // metallicity, edge by edge
-        if (t <= Zn && t < 32) {
-            const float y = (et.lgz[t] - s.th[7]) * (1.0f / s.th[8]);
-            const float dd = ((t < Zn) ? s.qb[t] : 0.0f) - ((t > 0) ? s.qb[t - 1] : 0.0f);
-            a[10] = phi_(y) * dd;
-            a[11] = phi_y(y) * dd;
-        }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-        for (int k = 0; k < SPS_NPARAM; ++k) a[k] += __shfl_xor_sync(kFull, a[k], o);
-    if (lane == 0)
-#pragma unroll
-        for (int k = 0; k < SPS_NPARAM; ++k) s.sums[warp][k] = a[k];
-    __syncthreads();
-    if (warp != 0) return;
-    float sv = 0.0f;
-    if (lane < SPS_NPARAM) sv = (s.sums[0][lane] + s.sums[1][lane]) + (s.sums[2][lane] + s.sums[3][lane]);
-    auto sum = [&](int k) { return __shfl_sync(kFull, sv, k); };
-    const float s_wp = sum(0), s_wm = sum(1), s_w0 = sum(2), s_w1 = sum(3), s_w2 = sum(4), s_d0 = sum(5), s_d1 = sum(6),
-                s_d2 = sum(7), s_mu = sum(8), s_sg = sum(9), s_gz = sum(10), s_gs = sum(11);
-    const float omf = 1.0f - fb, fa = fb * s_wp;
-    const float tT = tri_pdf(xT), kb = fb * Mf / (sig * D), isz = 1.0f / s.th[8];
-    const float out[SPS_NPARAM] = {s.gd[0], omf * s_w0 + fa * s_d0, omf * s_w1 + fa * s_d1, omf * s_w2 + fa * s_d2,
-                                   Mf * s_wp - s_wm, kb * (s_mu + s_wp * tT),
-                                   kb * (s_sg + s_wp * xT * tT) * (1.0f / 3.0f), s_gz * isz, s_gs * isz, s.gd[1],
-                                   s.gd[2], s.gd[3]};
+    // ---- through the SFH, burst and MDF weights
+    float out[SPS_NPARAM];
+    if (!few_adjoint(c, v, et, s.th, lT10, Mf, mi, pi, wb, s.sums, out)) return;
+    out[0] = s.gd[0];
+    out[9] = s.gd[1];
+    out[10] = s.gd[2];
+    out[11] = s.gd[3];
     float gk = 0.0f;
 #pragma unroll
     for (int k = 0; k < SPS_NPARAM; ++k)

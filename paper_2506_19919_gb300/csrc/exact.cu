@@ -18,11 +18,6 @@ namespace sps {
 
 namespace {
 
-__device__ __forceinline__ uint16_t f_to_bf16(float f) {
-    __nv_bfloat16 b = __float2bfloat16_rn(f);
-    return *reinterpret_cast<uint16_t*>(&b);
-}
-
 // ---------------------------------------------------------------- weights
 // W rows of the exact path, one row per warp: SFH, burst and MDF weights, then
 // W_k = w_i q_j as FP32, its TF32 halves, or BF16 scaled by 2^{e_i}.  Bound by
@@ -559,6 +554,8 @@ cudaError_t launch_exact_weights(const Consts& c, const Grid& grid, const Galaxi
                                  float* W32, uint16_t* Wbf, cudaStream_t s, const int32_t* pos_of,
                                  float* W32lo, float* keep, uint32_t* hull) {
     if (n <= 0) return cudaSuccess;
+    if (!c.mdf_age && n <= exact_few_rows())
+        return launch_weights_few(c, grid, g, theta, gal_idx, n, bf16, W32, Wbf, s, pos_of, W32lo, keep, hull);
     int blocks = 0;
     cudaError_t e;
     if (c.mdf_age) {
@@ -693,6 +690,8 @@ cudaError_t launch_exact_grad(const Consts& c, const Galaxies& g, const float* t
                               const float* keep, const int32_t* pos_of, int nsplit) {
     if (n <= 0) return cudaSuccess;
     if (!c.mdf_age && c.n_met <= kZnReg && keep) {
+        if (n <= exact_few_rows())
+            return launch_grad_few(c, g, theta, gal_idx, n, rowinfo, Wbar, grad_out, s, rowz, keep, pos_of, nsplit);
         int blocks = 0;
         const cudaError_t e = row_blocks(k_exact_grad_sep, 0, n, blocks);
         if (e != cudaSuccess) return e;

@@ -31,6 +31,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <cuda_bf16.h>
+
 #include "sps_internal.h"
 
 namespace sps {
@@ -98,6 +100,11 @@ __device__ __forceinline__ float tri_cdf(float x) {
 __device__ __forceinline__ float tri_pdf(float x) {
     float t = 1.0f - (x * x) * (1.0f / 9.0f);
     return (fabsf(x) <= 3.0f) ? (35.0f / 96.0f) * t * t * t : 0.0f;
+}
+
+__device__ __forceinline__ uint16_t f_to_bf16(float f) {
+    __nv_bfloat16 b = __float2bfloat16_rn(f);
+    return *reinterpret_cast<uint16_t*>(&b);
 }
 
 // ---------------------------------------------------------------- 3xTF32 split

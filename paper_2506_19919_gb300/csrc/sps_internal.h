@@ -153,6 +153,16 @@ cudaError_t launch_exact_weights(const Consts& c, const Grid& grid, const Galaxi
                                  float* keep = nullptr,              // with keep: the row's weight arrays
                                                                      // (keep_stride floats per row)
                                  uint32_t* hull = nullptr);          // with hull (zeroed): the row tiles' hulls
+// The same two for up to exact_few_rows() rows of the separable model (the
+// gradient with Zn <= 12 and keep), exact_few.cu; launch_exact_weights and
+// launch_exact_grad choose them.
+int64_t exact_few_rows();
+cudaError_t launch_weights_few(const Consts& c, const Grid& grid, const Galaxies& g, const float* theta,
+                               const int32_t* gal_idx, int64_t n, int bf16, float* W32, uint16_t* Wbf, cudaStream_t s,
+                               const int32_t* pos_of, float* W32lo, float* keep, uint32_t* hull);
+cudaError_t launch_grad_few(const Consts& c, const Galaxies& g, const float* theta, const int32_t* gal_idx, int64_t n,
+                            const float* rowinfo, const float* Wbar, float* grad_out, cudaStream_t s,
+                            const float* rowz, const float* keep, const int32_t* pos_of, int nsplit);
 // SIMT contractions (exact_simt.cu).  The forward writes nsplit slices of cJ
 // ([n][B][4] each; cJz [n][B][2]), the adjoint nsplit slices of Wbar ([n][k_pad]),
 // which the likelihood and gradient kernels add up in order; simt_*_split
