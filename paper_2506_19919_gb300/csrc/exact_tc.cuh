@@ -242,8 +242,11 @@ __device__ __forceinline__ uint8_t* carve(unsigned char* raw, Ctl*& ctl) {
 // Epilogue layout: 4 x n_groups x n_halves warps (fwd_shape).  A warp reads the TMEM lane
 // quarter q = (warp id mod 4) (32 rows) of each tile, for the bands of its group (<= NB, held in
 // registers) and one of n_halves (1, 2 or 3) parts of the tile's columns.  Rows arrive sorted by redshift (perm), so the 32 rows of a warp see
-// nearly the same band supports: a band is visited in a 32-column chunk only if
-// it overlaps the chunk in some lane.
+// nearly the same band supports: a band is visited in a group of 8 columns only if
+// its support reaches the group in some lane, and columns are tested against a
+// lane's own support only in groups that are not inside every lane's.  A row ends
+// at its own support whatever its neighbours: past it the weight is small, but under
+// steep dust the flux is not (6e-2 mag at A_V = 3, delta = -1, F_floor = 0, z = 2.9).
 // KZ also accumulates the redshift derivative of the band weights,
 // wb' = q_n T'((1+z) l_n), into cJz[row][b][2] = sum_n wb' S (1, E).
 template <int MAXT, int NB, int BN, bool TF, bool KZ>
@@ -330,14 +333,22 @@ k_fwd_tc(const __grid_constant__ TcMaps tm, const __grid_constant__ Consts c, co
             acc[k][0] = acc[k][1] = acc[k][2] = acc[k][3] = 0.0f;
             if (KZ) accz[k][0] = accz[k][1] = 0.0f;
         }
-        // warp-wide hull of each band's support (lanes without the band excluded):
-        // a group is visited for a band if the hull reaches it
-        uint32_t hxy[NB];                          // [lo, hi): lo | hi << 16
+        // lane k keeps band k's hull over the warp's rows (lanes without the band excluded)
+        // and the intersection of its supports; one ballot each per group of columns,
+        // where a word per band in every lane spilled (100,000 rows, six bands, BF16
+        // photometry 1.31 ms a call, 1.41 with words)
+        int2 hull_k = make_int2(0, 0), cut_k = make_int2(0, 0);
 #pragma unroll
         for (int k = 0; k < NB; ++k) {
             const int lo = (int)(sxy[k] & 0xffffu), hi = (int)(sxy[k] >> 16);
-            hxy[k] = __reduce_min_sync(0xffffffffu, (unsigned)(lo < hi ? lo : 0xffff)) |
-                     (__reduce_max_sync(0xffffffffu, (unsigned)(lo < hi ? hi : 0)) << 16);
+            const uint32_t h0 = __reduce_min_sync(0xffffffffu, (unsigned)(lo < hi ? lo : 0xffff));
+            const uint32_t h1 = __reduce_max_sync(0xffffffffu, (unsigned)(lo < hi ? hi : 0));
+            const uint32_t i0 = __reduce_max_sync(0xffffffffu, (unsigned)lo);
+            const uint32_t i1 = __reduce_min_sync(0xffffffffu, (unsigned)hi);
+            if (lane == k) {
+                hull_k = make_int2((int)h0, (int)h1);
+                cut_k = make_int2((int)i0, (int)i1);
+            }
         }
         bool has_tab = false;                      // a tabulated band in this warp's group
 #pragma unroll
@@ -408,12 +419,9 @@ k_fwd_tc(const __grid_constant__ TcMaps tm, const __grid_constant__ Consts c, co
                             tc::tmem_ld8_issue(taddr + (uint32_t)((h + 1) * CG), rn);
                             if (TF) tc::tmem_ld8_issue(taddr + (uint32_t)(BN + (h + 1) * CG), rc);
                         }
-                        uint32_t act = 0;                          // warp-uniform
-#pragma unroll
-                        for (int k = 0; k < NB; ++k) {
-                            if ((int)(hxy[k] & 0xffffu) < g0 + CG && (int)(hxy[k] >> 16) > g0) act |= 1u << k;
-                        }
+                        const uint32_t act = __ballot_sync(0xffffffffu, hull_k.x < g0 + CG && hull_k.y > g0);
                         if (act == 0u) continue;
+                        const uint32_t edges = __ballot_sync(0xffffffffu, cut_k.x > g0 || cut_k.y < g0 + CG);
                         float s0[CG], sE[CG], sEb[CG], sEd[CG], lm[CG];
 #pragma unroll
                         for (int jj = 0; jj < CG; ++jj) {
@@ -440,20 +448,19 @@ k_fwd_tc(const __grid_constant__ TcMaps tm, const __grid_constant__ Consts c, co
                                 const float gsv = gs[k] * 0.84932180028801904f;
                                 const float2 ngc = make_float2(-gc[k], -gc[k]), gs2 = make_float2(gsv, gsv);
                                 const bool gauss = gs[k] != 0.0f;
+                                const bool edge = (edges >> k) & 1u;
 #pragma unroll
                                 for (int jj = 0; jj < CG; jj += 2) {
-                                    // a Gaussian needs no range test: past its support (6 sigma) it
-                                    // adds, where a neighbouring row's support reaches, less than
-                                    // 2e-9 of the band's weight
-                                    float2 w;
+                                    float2 w = make_float2(1.0f, 1.0f);
                                     if (gauss) {
                                         const float2 u = __fmul2_rn(__fadd2_rn(make_float2(lm[jj], lm[jj + 1]), ngc), gs2);
                                         const float2 t = __fmul2_rn(u, u);
                                         w = make_float2(ex2_(-t.x), ex2_(-t.y));
-                                    } else {
+                                    }
+                                    if (edge) {                    // warp-uniform
                                         const int nn = g0 + jj;
-                                        w = make_float2(nn >= lo && nn < hi ? 1.0f : 0.0f,
-                                                        nn + 1 >= lo && nn + 1 < hi ? 1.0f : 0.0f);
+                                        w.x = nn >= lo && nn < hi ? w.x : 0.0f;
+                                        w.y = nn + 1 >= lo && nn + 1 < hi ? w.y : 0.0f;
                                     }
                                     p0 = __ffma2_rn(make_float2(s0[jj], s0[jj + 1]), w, p0);
                                     p1 = __ffma2_rn(make_float2(sE[jj], sE[jj + 1]), w, p1);

@@ -1,0 +1,70 @@
+"""Where a band ends: a Gaussian is integrated over |l - p0| < 6 s and no
+further, whatever other rows share a tensor-core tile, also where steep dust
+makes the spectrum rise by orders of magnitude past that limit.
+
+Bars: 3xTF32 and FP32 1e-4 mag and BF16 5e-3 mag against the FP64 oracle (an
+exponent of ~60 carries ~1e-5 relative rounding); the same row alone 2e-5 mag
+(another order of FP32 sums of such exponentials); gradients 1e-3 (BF16 3e-2) of the row's
+largest component."""
+import numpy as np
+import pytest
+
+import sps_workloads as W
+from oracle import sps as O
+
+pytestmark = pytest.mark.gpu
+
+
+def _flat(n_band, n_lam=1501):
+    """A table without spectral features, of order one (attenuated by 35 mag and
+    more, fluxes stay normal numbers), bands whose tails reach the far UV."""
+    rng = np.random.default_rng(3)
+    bands = W._gauss_bands(np.geomspace(3000.0, 9000.0, n_band))
+    t = W.make_tables(rng, 19, 7, n_lam, 91.0, 12000.0, bands)
+    t.ssp = np.repeat(t.ssp.mean(-1, keepdims=True), n_lam, -1) / t.ssp.mean()
+    return t
+
+
+def _cut_gaussians(monkeypatch):
+    """The oracle's Gaussians go on past 6 s; the library's end there."""
+    full = O.transmission
+
+    def cut(tables, lam_obs):
+        T = full(tables, lam_obs)
+        for b in np.flatnonzero(np.asarray(tables.band_kind) == W.BAND_GAUSS):
+            s = tables.band_p1[b] / (2.0 * np.sqrt(2.0 * np.log(2.0)))
+            T[..., b, :] *= ((lam_obs - tables.band_p0[b]).abs() < 6.0 * s).to(T.dtype)
+        return T
+
+    monkeypatch.setattr(O, "transmission", cut)
+
+
+@pytest.mark.parametrize("n_band", [2, 6, 8, 9, 17])
+def test_gaussian_support_under_steep_dust(n_band, monkeypatch):
+    import paper_2506_19919_gb300 as pkg
+    _cut_gaussians(monkeypatch)
+    t = _flat(n_band)
+    n = 64
+    z = np.linspace(0.3, 2.9, n).astype(np.float32).astype(np.float64)
+    th = W.prior_draw(np.random.default_rng(4), n)
+    th[:, 9], th[:, 10], th[:, 11] = 3.0, -1.0, 0.0              # A_V, delta, F_floor
+    ctx = pkg.Context(t)
+    ctx.set_galaxies(z, build_approx=False)
+    ref = O.photometry(th, z, t, "exact").numpy()
+    obs = (ref - 1.0).astype(np.float32).astype(np.float64)
+    sigma, mask = np.full(obs.shape, 0.05), np.full(n, (1 << n_band) - 1, np.uint32)
+    _, gr, _ = O.loglike_and_grad(th, z, t, obs, sigma, mask, "exact", wrt_z=True)
+    gr = gr.numpy()
+    scale = np.abs(gr).max(1, keepdims=True)
+    for prec, mtol, gtol in (("fp32", 1e-4, 1e-3), ("tf32x3", 1e-4, 1e-3), ("bf16", 5e-3, 3e-2)):
+        m = ctx.photometry(th, mode="exact", prec=prec).cpu().numpy()
+        assert np.abs(m - ref).max() < mtol, prec
+        for i in (0, 31, n - 1):
+            alone = ctx.photometry(th[i:i + 1], gal_idx=np.array([i], np.int32), mode="exact", prec=prec).cpu().numpy()
+            assert np.abs(alone - m[i]).max() < 2e-5, prec
+        ll, g = (x.cpu().numpy() for x in ctx.loglike_grad(th, obs, sigma, mask, mode="exact", prec=prec))
+        lz, gz = (x.cpu().numpy() for x in ctx.loglike_grad_z(th, obs, sigma, mask, mode="exact", prec=prec))
+        assert (np.abs(g - gr[:, :12]) / scale).max() < gtol, prec
+        assert (np.abs(g - gz[:, :12]) / scale).max() < 1e-3, prec
+        np.testing.assert_allclose(ll, lz, rtol=1e-3)
+    ctx.close()
