@@ -1367,6 +1367,10 @@ extern "C" sps_status sps_hmc_run(sps_ctx* ctx, const sps_hmc_config* cfg, const
         std::string gk = std::string(kb) + ":" + std::to_string(blocks) + ":" + std::to_string(cpw) + kc + ":" +
                          std::to_string(hp.sync_every) + ":" + std::to_string(main_end) + ":" +
                          std::to_string(blocks1);
+        // the captured launches hold the addresses of the galaxy tables, which another
+        // set_galaxies may have moved
+        const Galaxies tables = ctx->gal();
+        gk.append(reinterpret_cast<const char*>(&tables), sizeof(tables));
         if (!ctx->graph || gk != ctx->graph_key) {
             if (ctx->graph) {
                 cudaGraphExecDestroy(ctx->graph);
