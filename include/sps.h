@@ -78,7 +78,9 @@ typedef enum { SPS_EXACT = 0, SPS_APPROX = 1 } sps_mode;
  *             accumulation on the tensor cores (~1e-3 mag);
  *  SPS_TF32X3 FP32 operands split into TF32 halves, hi*hi + hi*lo + lo*hi on
  *             the tensor cores (~3e-5 mag, gradients ~1e-3: the tensor-core
- *             accumulation over the 1284-term contraction limits it). */
+ *             accumulation over the 1284-term contraction limits it).
+ * Grids of more than 65,535 wavelengths are contracted without the tensor cores
+ * (SPS_TF32X3 then in FP32). */
 typedef enum { SPS_FP32 = 0, SPS_BF16 = 1, SPS_TF32X3 = 2 } sps_prec;
 typedef enum { SPS_BAND_TOPHAT = 0, SPS_BAND_GAUSS = 1, SPS_BAND_TABLE = 2 } sps_band_kind;
 

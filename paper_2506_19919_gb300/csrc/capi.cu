@@ -601,8 +601,9 @@ static sps_status run_exact(sps_ctx* ctx, const float* theta, const int32_t* gid
     // tcgen05 for BF16 operands (SIMT when disabled) and for 3xTF32; FP32 is SIMT
     if (prec == SPS_TF32X3 && !ctx->use_tc) return fail(SPS_E_UNSUPPORTED, "3xTF32 needs the tensor cores");
     const int bf16 = prec == SPS_BF16 ? 1 : 0;
-    const bool tf = prec == SPS_TF32X3;
-    const bool tc = tf || (bf16 && ctx->use_tc);
+    const bool fits = c.n_lam <= kTcMaxLam;       // longer grids: the same operands in SIMT, FP32 for 3xTF32
+    const bool tf = prec == SPS_TF32X3 && fits;
+    const bool tc = tf || (bf16 && ctx->use_tc && fits);
     const int64_t chunk = tc ? (tf ? 65536 : 131072) : 32768;
     const int64_t rows = std::min<int64_t>(n, chunk);
     const int fsplit = tc ? tc_fwd_split(c, rows, tf) : simt_fwd_split(c, rows, 64);   // slices of the band sums

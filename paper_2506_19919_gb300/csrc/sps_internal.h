@@ -211,6 +211,8 @@ __host__ __device__ inline int64_t keep_stride(const Consts& c) { return (2 + 6 
 struct TcMaps {
     CUtensorMap a[2], b[2];
 };
+// Longest wavelength grid: the forward packs the two ends of a support in 16 bits each.
+constexpr int kTcMaxLam = 0xffff;
 int tc_fwd_columns(const Consts& c, bool tf);   // wavelengths per tile of the forward: box rows of its b maps
 size_t tc_adj_smem(bool tf);
 cudaError_t launch_fwd_tc(const TcMaps& tm, bool tf, const Consts& c, const Grid& grid, const Galaxies& g,

@@ -1,6 +1,7 @@
 """Where a band ends: a Gaussian is integrated over |l - p0| < 6 s and no
 further, whatever other rows share a tensor-core tile, also where steep dust
-makes the spectrum rise by orders of magnitude past that limit.
+makes the spectrum rise by orders of magnitude past that limit; and bands
+anywhere on a grid of more than 65,536 wavelengths.
 
 Bars: 3xTF32 and FP32 1e-4 mag and BF16 5e-3 mag against the FP64 oracle (an
 exponent of ~60 carries ~1e-5 relative rounding); the same row alone 2e-5 mag
@@ -67,4 +68,36 @@ def test_gaussian_support_under_steep_dust(n_band, monkeypatch):
         assert (np.abs(g - gr[:, :12]) / scale).max() < gtol, prec
         assert (np.abs(g - gz[:, :12]) / scale).max() < 1e-3, prec
         np.testing.assert_allclose(ll, lz, rtol=1e-3)
+    ctx.close()
+
+
+@pytest.mark.parametrize("kind", ["gauss", "table", "tophat"])
+def test_more_wavelengths_than_16_bits(kind):
+    """Bands on both sides of grid index 65,536 and across it."""
+    import paper_2506_19919_gb300 as pkg
+    rng = np.random.default_rng(5)
+    centres = np.array([6000.0, 10200.0, 11000.0]) * 1.05
+    bands = {"gauss": (np.full(3, W.BAND_GAUSS, np.int32), centres, centres / 60.0),
+             "tophat": (np.full(3, W.BAND_TOPHAT, np.int32), centres - 300.0, centres + 300.0)}.get(kind)
+    t = W.make_tables(rng, 6, 3, 70001, 900.0, 12000.0, bands or W._gauss_bands([5000.0]))
+    if kind == "table":
+        k, p0, p1, tn, tT = W.tabulated_bands(rng, [600.0, 1000.0, 1110.0, 1150.0])
+        t = W.with_bands(t, k, p0, p1, tn, tT)
+    n = 9
+    z = rng.uniform(0.03, 0.07, n).astype(np.float32).astype(np.float64)
+    th = W.prior_draw(rng, n)
+    ctx = pkg.Context(t)
+    ctx.set_galaxies(z, build_approx=False)
+    ref = O.photometry(th, z, t, "exact").numpy()
+    obs = (ref - 1.0).astype(np.float32).astype(np.float64)
+    sigma, mask = np.full(obs.shape, 0.05), np.full(n, 7, np.uint32)
+    _, gr, _ = O.loglike_and_grad(th, z, t, obs, sigma, mask, "exact")
+    gr = gr.numpy()
+    for prec, mtol, gtol in (("fp32", 2e-5, 1e-4), ("tf32x3", 1e-4, 1e-3), ("bf16", 5e-3, 3e-2)):
+        assert np.abs(ctx.photometry(th, mode="exact", prec=prec).cpu().numpy() - ref).max() < mtol, prec
+        _, g = ctx.loglike_grad(th, obs, sigma, mask, mode="exact", prec=prec)
+        assert (np.abs(g.cpu().numpy() - gr).max(1) / np.abs(gr).max(1)).max() < gtol, prec
+        if kind != "tophat":
+            _, gz = ctx.loglike_grad_z(th, obs, sigma, mask, mode="exact", prec=prec)
+            assert (np.abs(gz.cpu().numpy()[:, :12] - gr).max(1) / np.abs(gr).max(1)).max() < gtol, prec
     ctx.close()
