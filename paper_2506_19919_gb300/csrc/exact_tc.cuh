@@ -521,22 +521,42 @@ k_fwd_tc(const __grid_constant__ TcMaps tm, const __grid_constant__ Consts c, co
             tc::tc_fence_before();
             tc::mbar_arrive(&ctl->tempty[buf]);
         }
-        // the block's slice of cJ is zeroed before the launch; a (row, band) gets
-        // one addend per column part (the order of three moves at most the last bit)
-        if (valid && !ctl->abort) {
+        // the column parts' sums meet in the ring (every load was consumed before the
+        // last tile's products were complete) and are added in order, so that a
+        // call's bits do not depend on which warp is first; one store per (row, band)
+        // into the block's slice of cJ (100 rows, six bands, BF16: log L + gradient 119
+        // us a call, 126 with cJ cleared and four atomics per band and part)
+        constexpr bool kParts = MAXT <= 64 + 32 * 12 && (NB == 6 || MAXT <= 64 + 32 * 8);   // fwd_shape: else one
+        float4* meet = reinterpret_cast<float4*>(ring);          // [part - 1][NB][kTM]
+        float2* meetz = reinterpret_cast<float2*>(meet + (n_halves - 1) * NB * kTM);
+        if (kParts && half > 0) {
+#pragma unroll
+            for (int k = 0; k < NB; ++k) {
+                const int o = ((half - 1) * NB + k) * kTM + rl;
+                meet[o] = make_float4(acc[k][0], acc[k][1], acc[k][2], acc[k][3]);
+                if (KZ) meetz[o] = make_float2(accz[k][0], accz[k][1]);
+            }
+        }
+        if (kParts) asm volatile("bar.sync 1, %0;" ::"r"(epi_threads) : "memory");
+        if (half == 0 && valid && !ctl->abort) {
 #pragma unroll
             for (int k = 0; k < NB; ++k)
                 if (b0 + k < b_end) {
-                    float* o = cJ + (((int64_t)blockIdx.y * n + row) * B + b0 + k) * 4;
-                    atomicAdd(o + 0, acc[k][0]);
-                    atomicAdd(o + 1, acc[k][1]);
-                    atomicAdd(o + 2, acc[k][2]);
-                    atomicAdd(o + 3, acc[k][3]);
-                    if (KZ) {
-                        float* oz = cJz + (((int64_t)blockIdx.y * n + row) * B + b0 + k) * 2;
-                        atomicAdd(oz + 0, accz[k][0]);
-                        atomicAdd(oz + 1, accz[k][1]);
+                    float4 a = make_float4(acc[k][0], acc[k][1], acc[k][2], acc[k][3]);
+                    float2 az = make_float2(0.f, 0.f);
+                    if (KZ) az = make_float2(accz[k][0], accz[k][1]);
+                    for (int p = 1; kParts && p < n_halves; ++p) {
+                        const int o = ((p - 1) * NB + k) * kTM + rl;
+                        const float4 v = meet[o];
+                        a = make_float4(a.x + v.x, a.y + v.y, a.z + v.z, a.w + v.w);
+                        if (KZ) {
+                            const float2 vz = meetz[o];
+                            az = make_float2(az.x + vz.x, az.y + vz.y);
+                        }
                     }
+                    const int64_t o = ((int64_t)blockIdx.y * n + row) * B + b0 + k;
+                    reinterpret_cast<float4*>(cJ)[o] = a;
+                    if (KZ) reinterpret_cast<float2*>(cJz)[o] = az;
                 }
         }
     }
@@ -553,13 +573,13 @@ cudaError_t fwd_tc_launch(const TcMaps& tm, bool tf, const Consts& c, const Grid
     static_assert(kHullRows % kTM == 0, "a tile lies in one hull");
     const dim3 blocks((unsigned)((n + kTM - 1) / kTM), nsplit);
     const FwdShape sh = fwd_shape(c.n_band, tf);
+    // the parts' meeting place (16 + 8 bytes per row and band) fits the smallest ring
+    static_assert(2 * 6 * kTM * 24 <= Ring<192, kFwdStages<192, false>, false>::kBytes &&
+                      2 * 6 * kTM * 24 <= Ring<96, kFwdStages<96, true>, true>::kBytes &&
+                      8 * kTM * 24 <= Ring<256, kFwdStages<256, false>, false>::kBytes &&
+                      8 * kTM * 24 <= Ring<128, kFwdStages<128, true>, true>::kBytes, "ring too small");
     const int threads = 64 + 32 * 4 * sh.groups * sh.parts;
-    cudaError_t e = cudaMemsetAsync(cJ, 0, (size_t)nsplit * n * c.n_band * 4 * sizeof(float), s);
-    if (e != cudaSuccess) return e;
-    if (cJz) {
-        e = cudaMemsetAsync(cJz, 0, (size_t)nsplit * n * c.n_band * 2 * sizeof(float), s);
-        if (e != cudaSuccess) return e;
-    }
+    cudaError_t e;
     auto go = [&](auto kern, size_t ring) -> cudaError_t {
         const size_t smem = ring + 256 + kFwdConstBytes + 1024;
         cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
