@@ -574,10 +574,16 @@ cudaError_t launch_exact_weights(const Consts& c, const Grid& grid, const Galaxi
 
 // ---------------------------------------------------------------- redshift order
 // Rows bucketed by log(1 + z) of their galaxy (2048 buckets over [0, 2.5]),
-// so that the rows of a tensor-core tile see nearly the same band supports.
+// so that the rows of a tile see nearly the same band supports; by row index
+// within a bucket, because the tile a row falls into decides where its sums start
+// and the same call has to give the same bits.  A stable counting sort: the rows
+// in kZSegs segments at most, a bucket histogram of each, the histograms' running
+// sums over the segments, and in each segment the warps take their places in turn.
 constexpr int kZBuckets = 2048;
+constexpr int kZSegs = 128;
+constexpr int kZThreads = 1024;
 
-int zsort_buckets() { return kZBuckets; }
+size_t zsort_scratch() { return (size_t)kZBuckets * (kZSegs + 1); }
 
 namespace {
 __device__ __forceinline__ int zbucket(const Galaxies& g, const int32_t* gal_idx, int64_t row) {
@@ -586,34 +592,77 @@ __device__ __forceinline__ int zbucket(const Galaxies& g, const int32_t* gal_idx
     const float u = log1pf(fmaxf(z, 0.0f)) * ((float)kZBuckets / 2.5f);
     return (u < (float)(kZBuckets - 1)) ? (int)u : kZBuckets - 1;   // NaN goes last
 }
-__global__ void k_zcount(const Galaxies g, const int32_t* __restrict__ gal_idx, int64_t n, int32_t* counts) {
-    const int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (row < n) atomicAdd(&counts[zbucket(g, gal_idx, row)], 1);
+// Histogram of segment blockIdx.x into hist[segment][bucket]; also zeroes the
+// `extra` ints at `zero`.
+__global__ void __launch_bounds__(kZThreads) k_zcount(const Galaxies g, const int32_t* __restrict__ gal_idx, int64_t n,
+                                                      int64_t seg, int32_t* __restrict__ hist,
+                                                      int32_t* __restrict__ zero, int64_t extra) {
+    __shared__ int32_t h[kZBuckets];
+    for (int i = threadIdx.x; i < kZBuckets; i += kZThreads) h[i] = 0;
+    __syncthreads();
+    const int64_t r0 = (int64_t)blockIdx.x * seg, r1 = min(n, r0 + seg);
+    for (int64_t row = r0 + threadIdx.x; row < r1; row += kZThreads) atomicAdd(&h[zbucket(g, gal_idx, row)], 1);
+    for (int64_t i = (int64_t)blockIdx.x * kZThreads + threadIdx.x; i < extra; i += (int64_t)gridDim.x * kZThreads)
+        zero[i] = 0;
+    __syncthreads();
+    for (int i = threadIdx.x; i < kZBuckets; i += kZThreads) hist[(int64_t)blockIdx.x * kZBuckets + i] = h[i];
 }
-// Exclusive scan of the bucket counts in place (one block of 1024 threads).
-__global__ void __launch_bounds__(1024) k_zscan(int32_t* counts) {
-    __shared__ int32_t part[1024];
-    const int t = threadIdx.x;
-    const int a = counts[2 * t], b = counts[2 * t + 1];
+// One thread per bucket: hist becomes the rows of the bucket in the segments
+// before; total[bucket] all of them.
+__global__ void __launch_bounds__(64) k_zprefix(int segs, int32_t* __restrict__ hist, int32_t* __restrict__ total) {
+    const int b = blockIdx.x * 64 + threadIdx.x;
+    int32_t sum = 0;
+#pragma unroll 16
+    for (int s = 0; s < segs; ++s) {
+        const int32_t v = hist[(int64_t)s * kZBuckets + b];
+        hist[(int64_t)s * kZBuckets + b] = sum;
+        sum += v;
+    }
+    total[b] = sum;
+}
+// Rows of segment blockIdx.x to their places.
+__global__ void __launch_bounds__(kZThreads) k_zscatter(const Galaxies g, const int32_t* __restrict__ gal_idx, int64_t n,
+                                                        int64_t seg, const int32_t* __restrict__ hist,
+                                                        const int32_t* __restrict__ total, int32_t* __restrict__ perm,
+                                                        int32_t* __restrict__ pos_of) {
+    __shared__ int32_t cursor[kZBuckets], part[kZThreads];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    // exclusive scan of the totals, plus this segment's offset in each bucket
+    const int a = total[2 * t], b = total[2 * t + 1];
     part[t] = a + b;
     __syncthreads();
-    for (int o = 1; o < 1024; o <<= 1) {
+    for (int o = 1; o < kZThreads; o <<= 1) {
         const int v = (t >= o) ? part[t - o] : 0;
         __syncthreads();
         part[t] += v;
         __syncthreads();
     }
     const int base = part[t] - (a + b);
-    counts[2 * t] = base;
-    counts[2 * t + 1] = base + a;
-}
-__global__ void k_zscatter(const Galaxies g, const int32_t* __restrict__ gal_idx, int64_t n, int32_t* cursor,
-                           int32_t* __restrict__ perm, int32_t* __restrict__ pos_of) {
-    const int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (row >= n) return;
-    const int pos = atomicAdd(&cursor[zbucket(g, gal_idx, row)], 1);
-    perm[pos] = (int32_t)row;
-    pos_of[row] = pos;
+    const int32_t* hs = hist + (int64_t)blockIdx.x * kZBuckets;
+    cursor[2 * t] = base + hs[2 * t];
+    cursor[2 * t + 1] = base + a + hs[2 * t + 1];
+    __syncthreads();
+    const int64_t r0 = (int64_t)blockIdx.x * seg, r1 = min(n, r0 + seg);
+    for (int64_t c0 = r0; c0 < r1; c0 += kZThreads) {
+        const int64_t row = c0 + t;
+        const int key = row < r1 ? zbucket(g, gal_idx, row) : -1;
+        const uint32_t same = __match_any_sync(kFull, key);
+        const int rank = __popc(same & ((1u << lane) - 1u));
+        int pos = 0;
+        for (int w = 0; w < kZThreads / 32; ++w) {         // the warps in order
+            if (w == warp) {
+                const int at = key >= 0 ? cursor[key] : 0;
+                __syncwarp();
+                if (key >= 0 && rank == 0) cursor[key] = at + __popc(same);
+                pos = at + rank;
+            }
+            __syncthreads();
+        }
+        if (key >= 0) {
+            perm[pos] = (int32_t)row;
+            pos_of[row] = pos;
+        }
+    }
 }
 // The order of few rows in one launch: every row's position is the number of
 // rows before it in (z, row), counted against the keys in shared memory.  Also
@@ -645,20 +694,21 @@ __global__ void __launch_bounds__(kZFew) k_zorder_few(const Galaxies g, const in
 }  // namespace
 
 cudaError_t launch_zsort(const Galaxies& g, const int32_t* gal_idx, int64_t n, int32_t* perm,
-                         int32_t* pos_of, int32_t* counts, cudaStream_t s, int64_t extra) {
+                         int32_t* pos_of, int32_t* scratch, cudaStream_t s, int64_t extra) {
     if (n <= 0) return cudaSuccess;
-    static_assert(kZBuckets == 2 * 1024, "scan layout");
-    if (n <= kZFew) {          // one launch instead of four
-        k_zorder_few<<<1, (unsigned)((n + 31) / 32 * 32), 0, s>>>(g, gal_idx, (int)n, perm, pos_of, counts + kZBuckets,
-                                                                  (int)extra);
+    static_assert(kZBuckets == 2 * kZThreads, "scan layout");
+    int32_t* zero = scratch + zsort_scratch();
+    if (n <= kZFew) {          // one launch instead of three
+        k_zorder_few<<<1, (unsigned)((n + 31) / 32 * 32), 0, s>>>(g, gal_idx, (int)n, perm, pos_of, zero, (int)extra);
         return cudaGetLastError();
     }
-    cudaError_t e = cudaMemsetAsync(counts, 0, sizeof(int32_t) * (size_t)(kZBuckets + extra), s);
-    if (e != cudaSuccess) return e;
-    const unsigned blocks = (unsigned)((n + 255) / 256);
-    k_zcount<<<blocks, 256, 0, s>>>(g, gal_idx, n, counts);
-    k_zscan<<<1, 1024, 0, s>>>(counts);
-    k_zscatter<<<blocks, 256, 0, s>>>(g, gal_idx, n, counts, perm, pos_of);
+    const int64_t rounds = (n + (int64_t)kZThreads * kZSegs - 1) / ((int64_t)kZThreads * kZSegs);
+    const int64_t seg = rounds * kZThreads;                // rows per segment
+    const int segs = (int)((n + seg - 1) / seg);
+    int32_t* total = scratch + (size_t)kZBuckets * kZSegs;
+    k_zcount<<<segs, kZThreads, 0, s>>>(g, gal_idx, n, seg, scratch, zero, extra);
+    k_zprefix<<<kZBuckets / 64, 64, 0, s>>>(segs, scratch, total);
+    k_zscatter<<<segs, kZThreads, 0, s>>>(g, gal_idx, n, seg, scratch, total, perm, pos_of);
     return cudaGetLastError();
 }
 

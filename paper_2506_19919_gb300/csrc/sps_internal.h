@@ -228,12 +228,12 @@ cudaError_t launch_adj_tc(const TcMaps& tm, bool tf, const Consts& c, const Grid
 // writing its own slice of cJ / Wbar as in the SIMT contractions
 int tc_fwd_split(const Consts& c, int64_t n, bool tf);
 int tc_adj_split(const Consts& c, int64_t n);
-// Rows ordered by redshift (bucketed in log(1+z)): perm[pos] = row,
-// pos_of[row] = pos; counts is scratch of zsort_buckets() ints, zeroed with the
-// `extra` ints after it.
-int zsort_buckets();
+// Rows ordered by redshift (bucketed in log(1+z)) and row index: perm[pos] = row,
+// pos_of[row] = pos; scratch is zsort_scratch() ints and the `extra` ints after
+// them, which are zeroed.
+size_t zsort_scratch();
 cudaError_t launch_zsort(const Galaxies& g, const int32_t* gal_idx, int64_t n, int32_t* perm,
-                         int32_t* pos_of, int32_t* counts, cudaStream_t s, int64_t extra = 0);
+                         int32_t* pos_of, int32_t* scratch, cudaStream_t s, int64_t extra = 0);
 
 // Plain per-galaxy forward-mode path (comparison baseline).
 size_t plain_scratch_bytes_per_row(const Consts& c);
