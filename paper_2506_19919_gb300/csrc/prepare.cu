@@ -321,7 +321,7 @@ k_band_finish(const __grid_constant__ Consts c, const double* __restrict__ band_
 // and keeps its accuracy: the Gaussian argument is formed in double-float, the
 // weight uses the accurate expf, and FP32 partial sums of 32 terms are added
 // up in double-float (an FP64 addition per 32 FMAs would cost twice the FMAs).
-// 4,001 galaxies x 12 bands on the 107 x 12 x 5,994 grid: 3.0 ms (33 TFLOP/s of
+// 4,001 galaxies x 12 bands on the 107 x 12 x 5,994 grid: 3.1 ms (33 TFLOP/s of
 // the 97 GFLOP inside the supports), 11.8 ms with one galaxy per block.
 constexpr int kCsspChunk = 64;
 constexpr int kCsspThreads = 256;       // at most, per block
@@ -366,6 +366,10 @@ k_cssp(const __grid_constant__ Consts c, const Grid grid, const Galaxies gal, co
             lo = min(lo, sup[j].x);
             hi = max(hi, sup[j].y);
         }
+    // from a multiple of the 32-term partial sums, so that a galaxy's row of the table
+    // has the same bits whichever galaxies share its tile (an empty term adds 0; 2%
+    // more wavelengths than from the hull's own start, whose loop bounds would vary)
+    lo &= ~31;
     auto fill = [&](int n0, float (*w)[GT]) {
         for (int e = tid; e < kCsspChunk * GT; e += nt) {
             const int t = e / GT, j = e % GT, n = n0 + t;

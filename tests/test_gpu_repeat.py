@@ -69,7 +69,8 @@ def test_redshift_order_of_many_rows(zmax):
 
 
 def test_galaxy_set_built_again():
-    """The tables of a set are the same bits each time."""
+    """The tables of a set are the same bits each time, and a galaxy's row of
+    them does not depend on the others (sets of 16 and of 4 galaxies a block)."""
     ctx, rng, z, obs, sigma, mask = _context(4, 3000, True, zmax=3.0)
     th = torch.as_tensor(W.prior_draw(rng, 3000).astype(np.float32)).cuda()
     call = lambda: [ctx.photometry(th, mode="approx"),                                       # noqa: E731
@@ -79,6 +80,11 @@ def test_galaxy_set_built_again():
         ctx.set_galaxies(z, build_approx=True)
         for a, b in zip(first, call()):
             assert torch.equal(a, b)
+    for step in (2, 11):
+        ctx.set_galaxies(z[1::step].copy(), build_approx=True)
+        some = ctx.loglike_grad_z(th[1::step], obs[1::step], sigma[1::step], mask[1::step])
+        for a, b in zip(first[3:], some):
+            assert torch.equal(a[1::step], b)
     ctx.close()
 
 
