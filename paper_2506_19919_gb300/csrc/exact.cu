@@ -316,8 +316,11 @@ k_exact_vgen(const __grid_constant__ Consts c, const Grid grid, const Galaxies g
             const float2 pw = make_float2(ex2_(pa.x), ex2_(pa.y));
             const float2 base = __ffma2_rn(make_float2(kl.x, kl.y), pw, __fmul2_rn(eb2, dr));
             const float2 ea = __fmul2_rn(cA2, base);
-            const float2 F = __ffma2_rn(omf2, make_float2(ex2_(ea.x), ex2_(ea.y)), ff2);
-            v = __fmul2_rn(__fmul2_rn(F, make_float2(lq.z, lq.w)), sum);
+            float2 E;                                            // as dust_eval's
+            if (__any_sync(kFull, fminf(ea.x, ea.y) < -126.0f)) E = make_float2(exp2f(ea.x), exp2f(ea.y));
+            else E = make_float2(ex2_(ea.x), ex2_(ea.y));
+            const float2 F = __ffma2_rn(omf2, E, ff2);
+            v = __fmul2_rn(F, __fmul2_rn(make_float2(lq.z, lq.w), sum));
         }
         if (nn >= h.y) continue;                                 // the hull's end is a multiple of 32
         const int64_t o = pos * c.lam_pad + nn;

@@ -243,7 +243,7 @@ k_fwd_simt(const __grid_constant__ Consts c, const Grid grid, const Galaxies g, 
                         }
                         const float pw = expf_(rd.y * L4.z);
                         const float base = L4.y * pw + rd.w * L4.w;
-                        const float E = ex2_(-0.4f * kLog2_10f * rd.x * base);
+                        const float E = exp2f(-0.4f * kLog2_10f * rd.x * base);   // as dust_eval's
                         const float dterm = L4.y * pw * L4.z - (rd.w > 0.0f ? 1.9f * L4.w : 0.0f);
                         const float Sn = (j & 1) ? acc[i][j / 2].y : acc[i][j / 2].x;
                         const float S = Sn * wb;

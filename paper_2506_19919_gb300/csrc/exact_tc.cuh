@@ -429,7 +429,7 @@ k_fwd_tc(const __grid_constant__ TcMaps tm, const __grid_constant__ Consts c, co
                             lm[jj] = cstl[h * CG + jj];
                             const float ypw = L4.y * ex2_(dl2 * L4.z);      // k0 (l / l_V)^delta
                             const float base = fmaf(eb, L4.w, ypw);
-                            const float E = ex2_(cA * base);
+                            const float E = exp2f(cA * base);   // as dust_eval's
                             const float dterm = fmaf(ypw, L4.z, nd19 * L4.w);
                             s0[jj] = S[jj] * L4.x;
                             sE[jj] = s0[jj] * E;

@@ -60,7 +60,8 @@ __device__ __forceinline__ int lane_id() { return threadIdx.x & 31; }
 // more instructions each); here results under 2^-126 are 0.  Elsewhere the bits
 // are the same.  In the quadrature, dust and filter loops that is 4% of a sampler
 // run (11.63 -> 11.14 ms for 16,384 chains x 2 trajectories) and 7-12% of an
-// exact BF16 call.
+// exact BF16 call.  Not for 10^(-0.4 A): past 95 mag it is denormal, and with
+// F_floor = 0 all that is left of a band in the far UV (1% of an exact BF16 call).
 __device__ __forceinline__ float ex2_(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -140,7 +141,7 @@ __device__ __forceinline__ DustTerms dust_eval(float k0, float lnr, float drude,
     float pw = expf_(delta * lnr);
     float base = k0 * pw + eb * drude;
     float A = AV * (1.0f / 4.05f) * base;
-    float E = ex2_(-0.4f * kLog2_10f * A);
+    float E = exp2f(-0.4f * kLog2_10f * A);     // not ex2_: not 0 past 95 mag
     DustTerms d;
     d.F = ffl + (1.0f - ffl) * E;
     float g = (1.0f - ffl) * E * (-0.4f * kLn10f);

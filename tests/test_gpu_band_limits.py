@@ -1,7 +1,8 @@
 """Where a band ends: a Gaussian is integrated over |l - p0| < 6 s and no
 further, whatever other rows share a tensor-core tile, also where steep dust
 makes the spectrum rise by orders of magnitude past that limit; and bands
-anywhere on a grid of more than 65,536 wavelengths.
+anywhere on a grid of more than 65,536 wavelengths; and magnitudes where dust
+leaves less than 2^-126 of the flux.
 
 Bars: 3xTF32 and FP32 1e-4 mag and BF16 5e-3 mag against the FP64 oracle (an
 exponent of ~60 carries ~1e-5 relative rounding); the same row alone 2e-5 mag
@@ -9,6 +10,7 @@ exponent of ~60 carries ~1e-5 relative rounding); the same row alone 2e-5 mag
 largest component."""
 import numpy as np
 import pytest
+import torch
 
 import sps_workloads as W
 from oracle import sps as O
@@ -100,4 +102,37 @@ def test_more_wavelengths_than_16_bits(kind):
         if kind != "tophat":
             _, gz = ctx.loglike_grad_z(th, obs, sigma, mask, mode="exact", prec=prec)
             assert (np.abs(gz.cpu().numpy()[:, :12] - gr).max(1) / np.abs(gr).max(1)).max() < gtol, prec
+    ctx.close()
+
+
+@pytest.mark.parametrize("mode,prec", [("approx", "fp32"), ("exact", "fp32"), ("exact", "bf16"), ("exact", "tf32x3")])
+def test_deep_attenuation_stays_finite(mode, prec):
+    """A band attenuated by 97-108 mag with F_floor = 0: 10^(-0.4 A) is a
+    denormal FP32 number of nine bits or more (1e-3 relative), not zero."""
+    import paper_2506_19919_gb300 as pkg
+    rng = np.random.default_rng(3)
+    bands = (np.full(2, W.BAND_TOPHAT, np.int32), np.array([1940.0, 5000.0]), np.array([1960.0, 6000.0]))
+    t = W.make_tables(rng, 19, 7, 4001, 91.0, 12000.0, bands)
+    t.ssp = np.repeat(t.ssp.mean(-1, keepdims=True), 4001, -1) * (1e15 / t.ssp.mean())   # fluxes stay normal numbers
+    n = 140
+    z = np.full(n, 2.9, np.float32).astype(np.float64)
+    th = W.prior_draw(rng, n)
+    th[:, 10], th[:, 11] = -0.2, 0.0
+    rest = 1950.0 / 3.9 * 1e-4
+    k = O.calzetti_k0(torch.tensor(rest)).item() * (rest / 0.55) ** -0.2
+    k += O.bump_strength(torch.tensor(-0.2)).item() * O.drude_shape(torch.tensor(rest)).item()
+    th[:, 9] = rng.uniform(99.0, 106.0, n) * 4.05 / k
+    th = th.astype(np.float32).astype(np.float64)
+    ctx = pkg.Context(t)
+    ctx.set_galaxies(z, build_approx=True)
+    ref = O.photometry(th, z, t, mode).numpy()
+    m = ctx.photometry(th, mode=mode, prec=prec).cpu().numpy()
+    assert np.abs(m - ref).max() < 5e-3
+    if mode == "exact":            # all but F_floor, whose column is 10^40 and more
+        obs = (ref - 1.0).astype(np.float32).astype(np.float64)
+        sigma, mask = np.full(obs.shape, 0.05), np.full(n, 3, np.uint32)
+        _, gr, _ = O.loglike_and_grad(th, z, t, obs, sigma, mask, mode)
+        gr = gr.numpy()[:, :11]
+        _, g = ctx.loglike_grad(th, obs, sigma, mask, mode=mode, prec=prec)
+        assert (np.abs(g.cpu().numpy()[:, :11] - gr).max(1) / np.abs(gr).max(1)).max() < 3e-2
     ctx.close()
