@@ -335,7 +335,7 @@ k_cssp(const __grid_constant__ Consts c, const Grid grid, const Galaxies gal, co
     __shared__ int64_t gidx[GT];
     __shared__ int2 sup[GT];
     __shared__ Df crs[GT], inv[GT];
-    __shared__ float iopz[GT];
+    __shared__ Df istep;                   // 1 / s of a Gaussian, 1 / step of a table
     const int tid = threadIdx.x, nt = blockDim.x;
     const int b = blockIdx.y;
     const int kind = c.band_kind[b];
@@ -349,15 +349,14 @@ k_cssp(const __grid_constant__ Consts c, const Grid grid, const Galaxies gal, co
         gidx[tid] = g;
         sup[tid] = make_int2(0, 0);
         crs[tid] = inv[tid] = Df{0.f, 0.f};
-        iopz[tid] = 0.0f;
         if (g >= 0) {
             const double opz = 1.0 + (double)gal.z[g];
             sup[tid] = gal.support[(size_t)g * c.n_band + b];
             crs[tid] = df_from(band_p0[b] / opz);
             inv[tid] = df_from(opz / (kind == 1 ? band_p1[b] * kFwhmToSigma : band_p1[b]));
-            iopz[tid] = (float)(1.0 / opz);
         }
     }
+    if (tid == 31) istep = df_from(1.0 / (kind == 1 ? band_p1[b] * kFwhmToSigma : band_p1[b]));
     __syncthreads();
     int lo = c.n_lam, hi = 0;                                   // hull of the tile's supports
 #pragma unroll
@@ -398,8 +397,7 @@ k_cssp(const __grid_constant__ Consts c, const Grid grid, const Galaxies gal, co
                     } else {
                         tab_Tdf(grid.band_T + c.tab_off[b], grid.band_Tl + c.tab_off[b], c.tab_n[b], u, dT);
                     }
-                    // times inv / (1+z): 1 / s or 1 / step
-                    v = df_mul(df_mul(Df{Q.x, Q.y}, dT), df_mul_f(inv[j], iopz[j])).h;
+                    v = df_mul(df_mul(Df{Q.x, Q.y}, dT), istep).h;
                 }
             }
             w[t][j] = v;
