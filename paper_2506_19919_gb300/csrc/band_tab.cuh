@@ -14,7 +14,9 @@ namespace sps {
 // found inside the samples, and its slope dT/du (the segment holding u).
 __device__ __forceinline__ Df tab_Tdf(const float* __restrict__ Th, const float* __restrict__ Tl, int n, Df u,
                                       Df& slope) {
-    const int m = min(max((int)floorf(u.h), 0), n - 2);
+    // u just below an integer rounds up to it in u.h: the segment is the one before
+    const float fl = floorf(u.h);
+    const int m = min(max((int)fl - (u.h == fl && u.l < 0.0f ? 1 : 0), 0), n - 2);
     const Df f = two_sum(u.h - (float)m, u.l);
     const Df t0{__ldg(Th + m), __ldg(Tl + m)}, t1{__ldg(Th + m + 1), __ldg(Tl + m + 1)};
     slope = df_sub(t1, t0);
