@@ -22,6 +22,15 @@ namespace {
 constexpr int kWarpsRow = 8;
 constexpr int kWarpsRowZ = 6;
 
+// Tables of up to 32 kTilesSmall columns (20 x 4, 50 x 6) have kernels of their own,
+// unrolled for that many.  With the loops of the widest table / their own: 2,000 rows
+// of a 20 x 4 table with the redshift column 83 / 74 us, photometry with an
+// age-dependent MDF 52 / 45; 30,000 rows of a 50 x 6 table 555 / 461 and 288 / 230.
+// Wider tables keep the one loop: stopping it at the table's end in blocks of 10
+// column groups took 25,000 to 30,000 rows of a 107 x 12 table from 0.96 to 1.15 ms.
+constexpr int kTilesSmall = 10;
+
+template <int kTiles>
 __global__ void __launch_bounds__(32 * kWarpsRow, 2)
 k_approx_rows(const __grid_constant__ Consts c, const Galaxies g, const float* __restrict__ theta,
               int unbounded, const int32_t* __restrict__ gal_idx, int64_t n,
@@ -58,7 +67,7 @@ k_approx_rows(const __grid_constant__ Consts c, const Galaxies g, const float* _
         const int nb = fill_slots(c, g, ww.d, gi, bits, like ? mag_obs : nullptr, sigma,
                                   g.cssp + (size_t)gi * B * c.K, false);
         float gr[SPS_NPARAM];
-        double ll = eval_row(c, ww, g.bins + (size_t)gi * c.n_age, g.lnT[gi], g.lT10[gi], p, nb,
+        double ll = eval_row<false, kTiles>(c, ww, g.bins + (size_t)gi * c.n_age, g.lnT[gi], g.lT10[gi], p, nb,
                              like, grad, gr);
         if (mag_out && lane < nb) mag_out[row * B + ww.d.band[lane]] = (float)ww.d.mag[lane];
         if (ll_out && lane == 0) ll_out[row] = (float)ll;
@@ -82,6 +91,7 @@ k_approx_rows(const __grid_constant__ Consts c, const Galaxies g, const float* _
 
 // log L and d log L / d(theta, z) of the approximate path, one warp per row:
 // grad_out[row][13], the last column the derivative in the galaxy's redshift.
+template <int kTiles>
 __global__ void __launch_bounds__(32 * kWarpsRowZ, 2)
 k_approx_rows_z(const __grid_constant__ Consts c, const Galaxies g, const float* __restrict__ theta,
                 const int32_t* __restrict__ gal_idx, int64_t n, const float* __restrict__ mag_obs,
@@ -113,7 +123,7 @@ k_approx_rows_z(const __grid_constant__ Consts c, const Galaxies g, const float*
         const int nb = fill_slots(c, g, ww.d, gi, mask[gi] & all, mag_obs, sigma, g.cssp + gb0 * c.K, false);
         const ZRow zr{g.dcssp + gb0 * c.K, g.dzp + gb0, g.ddust + gb0, g.dtdz[gi]};
         float gr[NG];
-        const double ll = eval_row<true>(c, ww, g.bins + (size_t)gi * c.n_age, g.lnT[gi], g.lT10[gi], p,
+        const double ll = eval_row<true, kTiles>(c, ww, g.bins + (size_t)gi * c.n_age, g.lnT[gi], g.lT10[gi], p,
                                          nb, true, true, gr, &zr);
         if (lane == 0) {
             ll_out[row] = (float)ll;
@@ -191,10 +201,11 @@ cudaError_t launch_approx_rows(const Consts& c, const Galaxies& g, const float* 
                                double* logp_out, int* nonfinite, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     const int warps = row_warps(n, kWarpsRow);
-    cudaError_t e = cudaFuncSetAttribute(k_approx_rows, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    auto kern = c.K <= 32 * kTilesSmall ? k_approx_rows<kTilesSmall> : k_approx_rows<kKTileMax>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)(kWarpsRow * sizeof(WarpWork)));
     if (e != cudaSuccess) return e;
-    k_approx_rows<<<blocks_for(n, warps), 32 * warps, warps * sizeof(WarpWork), s>>>(
+    kern<<<blocks_for(n, warps), 32 * warps, warps * sizeof(WarpWork), s>>>(
         c, g, theta, theta_unbounded, gal_idx, n, mag_obs, sigma, mask, mag_out, loglike_out,
         grad_out, logp_out, nonfinite);
     return cudaGetLastError();
@@ -206,10 +217,11 @@ cudaError_t launch_approx_rows_z(const Consts& c, const Galaxies& g, const float
                                  float* grad_out, int* nonfinite, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
     const int warps = row_warps(n, kWarpsRowZ);
-    cudaError_t e = cudaFuncSetAttribute(k_approx_rows_z, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    auto kern = c.K <= 32 * kTilesSmall ? k_approx_rows_z<kTilesSmall> : k_approx_rows_z<kKTileMax>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)(kWarpsRowZ * sizeof(WarpWork)));
     if (e != cudaSuccess) return e;
-    k_approx_rows_z<<<blocks_for(n, warps), 32 * warps, warps * sizeof(WarpWork), s>>>(
+    kern<<<blocks_for(n, warps), 32 * warps, warps * sizeof(WarpWork), s>>>(
         c, g, theta, gal_idx, n, mag_obs, sigma, mask, loglike_out, grad_out, nonfinite);
     return cudaGetLastError();
 }

@@ -62,8 +62,9 @@ struct ZRow {
 // d.mag[slot] (FP64) and, if grad, the physical-parameter gradient into g[12]
 // (warp-uniform).  kZ (with like and grad): also d log L / dz into g[12] (13
 // entries), the explicit part (filter, zero point, lambda_eff, c_SSP(z)) plus
-// the part through t_obs(z) (age bins, M, burst clipping).
-template <bool kZ = false>
+// the part through t_obs(z) (age bins, M, burst clipping).  kTiles: 32-column
+// groups of a table row the loops are unrolled for (K <= 32 kTiles).
+template <bool kZ = false, int kTiles = kKTileMax>
 __device__ inline double eval_row(const Consts& c, WarpWork& ww, const float2* __restrict__ bins,
                            float lnT, float lT10, const RowParams& p, int nb, bool like,
                            bool grad, float* gout, const ZRow* zr = nullptr) {
@@ -78,11 +79,11 @@ __device__ inline double eval_row(const Consts& c, WarpWork& ww, const float2* _
     const bool nonsep = c.mdf_age != 0;
     if (nonsep) mdf_rows_fill(c, c.lgz_edge, p.th[7], p.th[8], s.u.kbuf);
     // ((age, metallicity) of a column is stepped along, not divided out)
-    float wreg[kKTileMax];
+    float wreg[kTiles];
     const int di = 32 / Zn, dj = 32 % Zn;
     int ki = lane / Zn, kj = lane % Zn;
 #pragma unroll
-    for (int t = 0; t < kKTileMax; ++t) {
+    for (int t = 0; t < kTiles; ++t) {
         int k = lane + 32 * t;
         wreg[t] = (k < K) ? s.w[ki] * (nonsep ? s.u.kbuf[k] : s.q[kj]) : 0.0f;
         ki += di;
@@ -108,7 +109,7 @@ __device__ inline double eval_row(const Consts& c, WarpWork& ww, const float2* _
         // predicate per column the loads of a row are in flight together
         float a = 0.0f;
 #pragma unroll
-        for (int t = 0; t < kKTileMax; ++t) {
+        for (int t = 0; t < kTiles; ++t) {
             a = fmaf(wreg[t], C[min(lane + 32 * t, K - 1)], a);
         }
         a = warp_sum(a);
@@ -117,7 +118,7 @@ __device__ inline double eval_row(const Consts& c, WarpWork& ww, const float2* _
             const float* Cd = zr->dcssp + (size_t)d.band[sl] * K;
             float b = 0.0f;
 #pragma unroll
-            for (int t = 0; t < kKTileMax; ++t) {
+            for (int t = 0; t < kTiles; ++t) {
                 b = fmaf(wreg[t], Cd[min(lane + 32 * t, K - 1)], b);
             }
             b = warp_sum(b);
@@ -174,19 +175,19 @@ __device__ inline double eval_row(const Consts& c, WarpWork& ww, const float2* _
     gff = warp_sum(gff);
     __syncwarp();
     // v_k = sum_b (gamma_b / S_b) c_SSP[b][k], band by band, a row's loads together
-    float v[kKTileMax];
+    float v[kTiles];
 #pragma unroll
-    for (int t = 0; t < kKTileMax; ++t) v[t] = 0.0f;
+    for (int t = 0; t < kTiles; ++t) v[t] = 0.0f;
     for (int sl = 0; sl < nb; ++sl) {
         const float* C = d.ptr[sl];
         const float gb = s.slot_g[sl];
 #pragma unroll
-        for (int t = 0; t < kKTileMax; ++t) {
+        for (int t = 0; t < kTiles; ++t) {
             v[t] = fmaf(gb, C[min(lane + 32 * t, K - 1)], v[t]);
         }
     }
 #pragma unroll
-    for (int t = 0; t < kKTileMax; ++t) {
+    for (int t = 0; t < kTiles; ++t) {
         int k = lane + 32 * t;
         if (k < K) s.u.kbuf[k] = v[t];
     }
