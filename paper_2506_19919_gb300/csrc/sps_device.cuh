@@ -243,12 +243,12 @@ __device__ __forceinline__ int panel_count(float f) {
 //   u < 0:  hh = e^{(beta+1)u} r,  r = 1 / (1 + e^{(alpha+beta)u}),  hh P = 1 - r, hh Q = r
 //   u >= 0: hh = e^{(1-alpha)u} r, r = 1 / (1 + e^{-(alpha+beta)u}), hh P = r,     hh Q = 1 - r
 // so that dhh/dalpha = -u hh (hh P), dhh/dbeta = u hh (hh Q) and
-// alpha P - beta Q = (alpha hhP - beta hhQ) / hh.  kPack takes the nodes in pairs
+// alpha P - beta Q = (alpha hhP - beta hhQ) / hh.  All of it times 2^off.  kPack takes the nodes in pairs
 // with packed FP32x2 arithmetic (faster in the HMC team kernel, slower in the
 // one-row-per-warp kernels, which keep the scalar loop).
 template <int N, bool kPack = false>
 __device__ __forceinline__ void gl_panel(const float* __restrict__ gx, const float* __restrict__ gw,
-                                         float hp, float xc, float alpha, float beta, bool grad,
+                                         float hp, float xc, float alpha, float beta, float off, bool grad,
                                          float& v0, float& v1, float& v2, float& v3) {
     const float kL2E = 1.4426950408889634f;
     const float cneg = (beta + 1.0f) * kL2E, cpos = (1.0f - alpha) * kL2E, cs = -(alpha + beta) * kL2E;
@@ -261,7 +261,7 @@ __device__ __forceinline__ void gl_panel(const float* __restrict__ gx, const flo
         for (int q = 0; q + 1 < N; q += 2) {
             const float2 uu = __ffma2_rn(hp2, make_float2(gx[q], gx[q + 1]), xc2);
             const bool px = uu.x >= 0.0f, py = uu.y >= 0.0f;
-            const float2 Ea = __fmul2_rn(uu, make_float2(px ? cpos : cneg, py ? cpos : cneg));
+            const float2 Ea = __ffma2_rn(uu, make_float2(px ? cpos : cneg, py ? cpos : cneg), make_float2(off, off));
             const float2 Ra = __fmul2_rn(make_float2(fabsf(uu.x), fabsf(uu.y)), make_float2(cs, cs));
             const float2 E = make_float2(ex2_(Ea.x), ex2_(Ea.y));
             const float2 R = make_float2(ex2_(Ra.x), ex2_(Ra.y));
@@ -283,7 +283,7 @@ __device__ __forceinline__ void gl_panel(const float* __restrict__ gx, const flo
             const int q = N - 1;
             const float uu = fmaf(hp, gx[q], xc);
             const bool pos = uu >= 0.0f;
-            const float E = ex2_(uu * (pos ? cpos : cneg));
+            const float E = ex2_(fmaf(uu, pos ? cpos : cneg, off));
             const float R = ex2_(fabsf(uu) * cs);
             const float r = rcp_(1.0f + R);
             const float wh = gw[q] * hp * E * r;
@@ -308,7 +308,7 @@ __device__ __forceinline__ void gl_panel(const float* __restrict__ gx, const flo
         for (int q = 0; q < N; ++q) {
             const float uu = fmaf(hp, gx[q], xc);
             const bool pos = uu >= 0.0f;
-            const float E = ex2_(uu * (pos ? cpos : cneg));
+            const float E = ex2_(fmaf(uu, pos ? cpos : cneg, off));
             const float R = ex2_(fabsf(uu) * cs);
             const float r = rcp_(1.0f + R);
             const float wh = gw[q] * hp * E * r;                      // w hh
@@ -326,10 +326,10 @@ __device__ __forceinline__ void gl_panel(const float* __restrict__ gx, const flo
 }
 __device__ __forceinline__ void gl_panel_any(int n, const float* __restrict__ gx,
                                              const float* __restrict__ gw, float hp, float xc,
-                                             float alpha, float beta, bool grad, float& v0,
+                                             float alpha, float beta, float off, bool grad, float& v0,
                                              float& v1, float& v2, float& v3) {
 #pragma unroll 1
-    for (int q = 0; q < n; ++q) gl_panel<1>(gx + q, gw + q, hp, xc, alpha, beta, grad, v0, v1, v2, v3);
+    for (int q = 0; q < n; ++q) gl_panel<1>(gx + q, gw + q, hp, xc, alpha, beta, off, grad, v0, v1, v2, v3);
 }
 
 // Fills v.m and (if grad) v.dm0..2; returns M = sum_i m_i (FP64).
@@ -361,6 +361,11 @@ __device__ __forceinline__ void sfh_bins_raw(const Consts& c, const AgeView& v, 
     const float ipw = 1.0f / pw;
     const int G = c.gl_order;
     const int o2 = min(2, G), o3 = min(3, G);
+    // a history that peaks long after t_obs has hh = e^{(beta+1)u} far below 1 in every
+    // bin; below 2^-64 at t_obs it is integrated times 2^64, so that nothing that
+    // counts comes near 2^-126, where ex2_ ends
+    const bool faint = bp1 * (lnT - lntau) < -44.4f;
+    const float off = faint ? 64.0f : 0.0f, sc = faint ? 0x1p-64f : 1.0f, tau_sc = tau * sc;
     // Pass 1, bins i = lane + 32 k: panel layout; a bin that fits one panel is
     // integrated here, a bin of several panels is queued for pass 2.
     int base = 0;                               // panels queued so far (warp-uniform)
@@ -402,20 +407,20 @@ __device__ __forceinline__ void sfh_bins_raw(const Consts& c, const AgeView& v, 
         if (oc > 0 && ord > 0) {
             const float xc = x0 - lntau;
             if (oc <= 2)
-                gl_panel<2, kPack>(c.gl2_x, c.gl2_w, hp, xc, alpha, beta, grad, v0, v1, v2, v3);
+                gl_panel<2, kPack>(c.gl2_x, c.gl2_w, hp, xc, alpha, beta, off, grad, v0, v1, v2, v3);
             else if (oc == 3)
-                gl_panel<3, kPack>(c.gl3_x, c.gl3_w, hp, xc, alpha, beta, grad, v0, v1, v2, v3);
+                gl_panel<3, kPack>(c.gl3_x, c.gl3_w, hp, xc, alpha, beta, off, grad, v0, v1, v2, v3);
             else if (oc == 6)
-                gl_panel<6, kPack>(c.gl_x, c.gl_w, hp, xc, alpha, beta, grad, v0, v1, v2, v3);
+                gl_panel<6, kPack>(c.gl_x, c.gl_w, hp, xc, alpha, beta, off, grad, v0, v1, v2, v3);
             else
-                gl_panel_any(G, c.gl_x, c.gl_w, hp, xc, alpha, beta, grad, v0, v1, v2, v3);
+                gl_panel_any(G, c.gl_x, c.gl_w, hp, xc, alpha, beta, off, grad, v0, v1, v2, v3);
         }
         if (i < A) {
-            v.m[i] = v0 * tau;
+            v.m[i] = v0 * tau_sc;
             if (grad) {
-                v.dm0[i] = v1;
-                v.dm1[i] = v2 * tau;
-                v.dm2[i] = v3 * tau;
+                v.dm0[i] = v1 * sc;
+                v.dm1[i] = v2 * tau_sc;
+                v.dm2[i] = v3 * tau_sc;
             }
         }
         // queue the panels of multi-panel bins: exclusive scan of their counts (most
@@ -465,9 +470,9 @@ __device__ __forceinline__ void sfh_bins_raw(const Consts& c, const AgeView& v, 
             const float hp = inf.y;
             const float xc = inf.x + 2.0f * (float)(p - __float_as_int(inf.z)) * hp - lntau;
             if (G == 6)
-                gl_panel<6, kPack>(c.gl_x, c.gl_w, hp, xc, alpha, beta, grad, v0, v1, v2, v3);
+                gl_panel<6, kPack>(c.gl_x, c.gl_w, hp, xc, alpha, beta, off, grad, v0, v1, v2, v3);
             else
-                gl_panel_any(G, c.gl_x, c.gl_w, hp, xc, alpha, beta, grad, v0, v1, v2, v3);
+                gl_panel_any(G, c.gl_x, c.gl_w, hp, xc, alpha, beta, off, grad, v0, v1, v2, v3);
         }
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -482,11 +487,11 @@ __device__ __forceinline__ void sfh_bins_raw(const Consts& c, const AgeView& v, 
         }
         const int bnext = __shfl_down_sync(kFull, bin, 1);
         if (bin >= 0 && (lane == 31 || bnext != bin)) {
-            v.m[bin] += v0 * tau;
+            v.m[bin] += v0 * tau_sc;
             if (grad) {
-                v.dm0[bin] += v1;
-                v.dm1[bin] += v2 * tau;
-                v.dm2[bin] += v3 * tau;
+                v.dm0[bin] += v1 * sc;
+                v.dm1[bin] += v2 * tau_sc;
+                v.dm2[bin] += v3 * tau_sc;
             }
         }
         __syncwarp();
