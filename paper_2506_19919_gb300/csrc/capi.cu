@@ -494,7 +494,6 @@ sps_status sps_create(sps_ctx** out, const sps_tables* t, const sps_config* cfg_
         (e = upload(ctx->ssp_t, st32.data(), st32.size() * 4)) != cudaSuccess ||
         (e = upload(ctx->ssp_bf, sbf.data(), sbf.size() * 2)) != cudaSuccess ||
         (e = upload(ctx->ssp_t_bf, stbf.data(), stbf.size() * 2)) != cudaSuccess ||
-        (e = upload(ctx->row_scale, rscale.data(), rscale.size() * 4)) != cudaSuccess ||
         (e = upload(ctx->col_scale, cscale.data(), cscale.size() * 4)) != cudaSuccess ||
         (e = upload(ctx->age_edges, edges.data(), edges.size() * 8)) != cudaSuccess ||
         (e = upload(ctx->bp0, t->band_p0, sizeof(double) * B)) != cudaSuccess ||

@@ -69,7 +69,7 @@ struct sps_ctx {
     double gl_x[sps::kMaxGL], gl_w[sps::kMaxGL];
     std::vector<double> band_p0, band_p1;
     // tables
-    DevBuf lam64, lam32, lamc, lamp, lamd, lamdq, gl32, ssp, ssp_t, ssp_bf, ssp_t_bf, row_scale, col_scale, age_edges, bp0, bp1;
+    DevBuf lam64, lam32, lamc, lamp, lamd, lamdq, gl32, ssp, ssp_t, ssp_bf, ssp_t_bf, col_scale, age_edges, bp0, bp1;
     DevBuf ssp_hi, ssp_lo, ssp_t_hi, ssp_t_lo;   // 3xTF32 halves of the FP32 tables
     DevBuf tabT, tabTl;                          // tabulated transmission samples, high and low parts
     // galaxies
@@ -112,7 +112,6 @@ struct sps_ctx {
         g.ssp_t = ssp_t.as<float>();
         g.ssp_bf = ssp_bf.as<uint16_t>();
         g.ssp_t_bf = ssp_t_bf.as<uint16_t>();
-        g.row_scale = row_scale.as<float>();
         g.col_scale = col_scale.as<float>();
         g.band_T = tabT.as<float>();
         g.band_Tl = tabTl.as<float>();
@@ -143,7 +142,7 @@ struct sps_ctx {
         if (join) cudaEventDestroy(join);
         if (side) cudaStreamDestroy(side);
         if (flags) cudaFreeHost(flags);
-        DevBuf* all[] = {&lam64, &lam32, &lamc, &lamp, &lamd, &lamdq, &gl32, &prep, &ssp, &ssp_t, &ssp_bf, &ssp_t_bf, &row_scale, &col_scale,
+        DevBuf* all[] = {&lam64, &lam32, &lamc, &lamp, &lamd, &lamdq, &gl32, &prep, &ssp, &ssp_t, &ssp_bf, &ssp_t_bf, &col_scale,
                          &age_edges, &bp0, &bp1, &gz, &glnT, &glT10, &gbins, &gzp, &gsup, &ggauss,
                          &gcssp, &gdust, &gdtdz, &gdzp, &gddust, &gdcssp, &cJz, &rowz, &nonfinite, &queue, &err, &W, &V, &Wbar, &cJ, &gbar,
                          &rowinfo, &tcerr, &plainT, &plainC, &hmcm, &pst, &pth, &pll, &pgr,

@@ -256,7 +256,7 @@ k_exact_vgen(const __grid_constant__ Consts c, const Grid grid, const Galaxies g
     __shared__ int2 sp[kMaxBands];
     const int64_t pos = blockIdx.x;
     if (pos >= n) return;
-    const int64_t row = perm ? (int64_t)perm[pos] : pos;
+    const int64_t row = perm[pos];
     const int2 h = row_hull(c, hull, pos);
     const int B = c.n_band;
     int64_t gi = gal_idx ? (int64_t)gal_idx[row] : row;

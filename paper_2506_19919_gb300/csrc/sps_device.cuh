@@ -79,10 +79,9 @@ __device__ __forceinline__ float expf_(float x) { return ex2_(x * 1.442695040888
 // range, the hull of their band supports.  k_weights collects it per kHullRows
 // positions as (max of n_lam - lo, max of hi), from zeroed memory; row_hull
 // gives the range of the tile holding position pos, widened to multiples of 64
-// inside the padded grid (never empty; the whole grid without a hull).
+// inside the padded grid (never empty).
 constexpr int kHullRows = 128;
 __device__ __forceinline__ int2 row_hull(const Consts& c, const uint32_t* __restrict__ hull, int64_t pos) {
-    if (!hull) return make_int2(0, c.lam_pad);
     const uint2 h = reinterpret_cast<const uint2*>(hull)[pos / kHullRows];
     const int lo = c.n_lam - (int)h.x, hi = (int)h.y;
     if (hi <= lo) return make_int2(0, min(64, c.lam_pad));

@@ -72,7 +72,6 @@ struct Grid {
     const float* ssp;        // [k_pad][lam_pad] SSP table, FP32 (zero padded)
     const uint16_t* ssp_bf;  // [k_pad][lam_pad] SSP table, BF16 bits, row-scaled by 2^-e_i
     const uint16_t* ssp_t_bf;// [lam_pad][k_pad] transposed BF16 row-scaled
-    const float* row_scale;  // [A] 2^e_i
     const float* col_scale;  // [k_pad] 2^e_i of column k = i Zn + j, 0 past K
     const float* band_T;     // tabulated transmission samples, all TABLE bands (FP32)
     const float* band_Tl;    // their low parts, sample = T + Tl (per-galaxy set-up kernels)
@@ -187,9 +186,9 @@ cudaError_t launch_exact_like(const Consts& c, const Galaxies& g, const float* t
 cudaError_t launch_exact_vgen(const Consts& c, const Grid& grid, const Galaxies& g,
                               const float* theta, const int32_t* gal_idx, int64_t n,
                               const float* gbar, float* V32, uint16_t* Vbf, cudaStream_t s,
-                              float* V32lo = nullptr,    // with V32lo: V32 = TF32 hi, V32lo = lo
-                              const int32_t* perm = nullptr,      // the row at each position of V
-                              const uint32_t* hull = nullptr);    // v inside the row tiles' hulls only
+                              float* V32lo,              // if not null: V32 = TF32 hi, V32lo = lo
+                              const int32_t* perm,       // the row at each position of V
+                              const uint32_t* hull);     // v inside the row tiles' hulls only
 cudaError_t launch_exact_adj(const Consts& c, const Grid& grid, int64_t n, int bf16, const float* V32,
                              const uint32_t* hull, float* Wbar, int nsplit, cudaStream_t s);
 cudaError_t launch_exact_grad(const Consts& c, const Galaxies& g, const float* theta,
