@@ -533,7 +533,7 @@ sps_status sps_destroy(sps_ctx* ctx) {
 // The c_SSP table (deriv 0) or its redshift derivative, galaxies in redshift order.
 static sps_status build_cssp(sps_ctx* ctx, float* out, int deriv, cudaStream_t s) {
     const int64_t G = ctx->n_gal;
-    CK(ctx->zperm.reserve(sizeof(int32_t) * (2 * (size_t)G + zsort_scratch())));
+    CK(ctx->zperm.reserve(sizeof(int32_t) * (2 * (size_t)G + zsort_scratch(G))));
     int32_t* perm = ctx->zperm.as<int32_t>();
     CK(launch_zsort(ctx->gal(), nullptr, G, perm, perm + G, perm + 2 * G, s));
     CK(launch_cssp(ctx->c, ctx->grid(), ctx->gal(), perm, ctx->bp0.as<double>(), ctx->bp1.as<double>(), out, s,
@@ -614,11 +614,11 @@ static sps_status run_exact(sps_ctx* ctx, const float* theta, const int32_t* gid
     CK(ctx->gbar.reserve((size_t)rows * c.n_band * 4));
     // redshift order of the rows, the sort's scratch, row-tile hulls
     const int64_t hulls = 2 * ((rows + 127) / 128);
-    CK(ctx->zperm.reserve(sizeof(int32_t) * (2 * (size_t)rows + 2 + zsort_scratch() + (size_t)hulls)));
+    CK(ctx->zperm.reserve(sizeof(int32_t) * (2 * (size_t)rows + 2 + zsort_scratch(rows) + (size_t)hulls)));
     int32_t* perm = ctx->zperm.as<int32_t>();
     int32_t* pos_of = perm + rows;
     int32_t* zscratch = perm + 2 * ((rows + 1) / 2 * 2);
-    uint32_t* hull = reinterpret_cast<uint32_t*>(zscratch + zsort_scratch());
+    uint32_t* hull = reinterpret_cast<uint32_t*>(zscratch + zsort_scratch(rows));
     if (grad_out) {
         CK(ctx->V.reserve((size_t)rows * c.lam_pad * 4));
         CK(ctx->Wbar.reserve((size_t)asplit * rows * c.k_pad * 4));
@@ -658,7 +658,7 @@ static sps_status run_exact(sps_ctx* ctx, const float* theta, const int32_t* gid
             if (gv.dcssp) gv.dcssp += r0 * c.n_band * c.K;
             gv.n = m;
         }
-        CK(launch_zsort(gv, gi, m, perm, pos_of, zscratch, s, hulls));
+        CK(launch_zsort(gv, gi, m, perm, pos_of, zscratch, s, reinterpret_cast<int32_t*>(hull), hulls));
         CK(launch_exact_weights(c, grid, gv, th, gi, m, bf16, ctx->W.as<float>(), ctx->W.as<uint16_t>(), s,
                                 pos_of, tf ? ctx->Wlo.as<float>() : nullptr, keep, hull));
         if (tc) {

@@ -585,8 +585,19 @@ cudaError_t launch_exact_weights(const Consts& c, const Grid& grid, const Galaxi
 constexpr int kZBuckets = 2048;
 constexpr int kZSegs = 128;
 constexpr int kZThreads = 1024;
+constexpr int kZFew = 1024;            // up to here the order takes one launch and no scratch
 
-size_t zsort_scratch() { return (size_t)kZBuckets * (kZSegs + 1); }
+// Rows per segment, a multiple of kZThreads.
+static int64_t zsort_seg(int64_t n) {
+    return (n + (int64_t)kZThreads * kZSegs - 1) / ((int64_t)kZThreads * kZSegs) * kZThreads;
+}
+// Grows with the rows up to a chunk's 131,072 (24 KB for 1,025, 1 MB), so that a
+// chunk's buffer serves the last, shorter one; a megabyte for every call added 100 us
+// to the first call of a context.
+size_t zsort_scratch(int64_t n) {
+    if (n <= kZFew) return 0;
+    return (size_t)kZBuckets * (size_t)((n + zsort_seg(n) - 1) / zsort_seg(n) + 1);
+}
 
 namespace {
 __device__ __forceinline__ int zbucket(const Galaxies& g, const int32_t* gal_idx, int64_t row) {
@@ -670,7 +681,6 @@ __global__ void __launch_bounds__(kZThreads) k_zscatter(const Galaxies g, const 
 // The order of few rows in one launch: every row's position is the number of
 // rows before it in (z, row), counted against the keys in shared memory.  Also
 // zeroes the `extra` ints at `zero`.
-constexpr int kZFew = 1024;
 __global__ void __launch_bounds__(kZFew) k_zorder_few(const Galaxies g, const int32_t* __restrict__ gal_idx, int n,
                                                       int32_t* __restrict__ perm, int32_t* __restrict__ pos_of,
                                                       int32_t* __restrict__ zero, int extra) {
@@ -697,18 +707,16 @@ __global__ void __launch_bounds__(kZFew) k_zorder_few(const Galaxies g, const in
 }  // namespace
 
 cudaError_t launch_zsort(const Galaxies& g, const int32_t* gal_idx, int64_t n, int32_t* perm,
-                         int32_t* pos_of, int32_t* scratch, cudaStream_t s, int64_t extra) {
+                         int32_t* pos_of, int32_t* scratch, cudaStream_t s, int32_t* zero, int64_t extra) {
     if (n <= 0) return cudaSuccess;
     static_assert(kZBuckets == 2 * kZThreads, "scan layout");
-    int32_t* zero = scratch + zsort_scratch();
     if (n <= kZFew) {          // one launch instead of three
         k_zorder_few<<<1, (unsigned)((n + 31) / 32 * 32), 0, s>>>(g, gal_idx, (int)n, perm, pos_of, zero, (int)extra);
         return cudaGetLastError();
     }
-    const int64_t rounds = (n + (int64_t)kZThreads * kZSegs - 1) / ((int64_t)kZThreads * kZSegs);
-    const int64_t seg = rounds * kZThreads;                // rows per segment
+    const int64_t seg = zsort_seg(n);
     const int segs = (int)((n + seg - 1) / seg);
-    int32_t* total = scratch + (size_t)kZBuckets * kZSegs;
+    int32_t* total = scratch + (size_t)kZBuckets * segs;
     k_zcount<<<segs, kZThreads, 0, s>>>(g, gal_idx, n, seg, scratch, zero, extra);
     k_zprefix<<<kZBuckets / 64, 64, 0, s>>>(segs, scratch, total);
     k_zscatter<<<segs, kZThreads, 0, s>>>(g, gal_idx, n, seg, scratch, total, perm, pos_of);

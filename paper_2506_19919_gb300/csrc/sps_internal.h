@@ -228,11 +228,12 @@ cudaError_t launch_adj_tc(const TcMaps& tm, bool tf, const Consts& c, const Grid
 int tc_fwd_split(const Consts& c, int64_t n, bool tf);
 int tc_adj_split(const Consts& c, int64_t n);
 // Rows ordered by redshift (bucketed in log(1+z)) and row index: perm[pos] = row,
-// pos_of[row] = pos; scratch is zsort_scratch() ints and the `extra` ints after
-// them, which are zeroed.
-size_t zsort_scratch();
+// pos_of[row] = pos; scratch is zsort_scratch(n) ints; the `extra` ints at
+// `zero` are zeroed on the way.
+size_t zsort_scratch(int64_t n);
 cudaError_t launch_zsort(const Galaxies& g, const int32_t* gal_idx, int64_t n, int32_t* perm,
-                         int32_t* pos_of, int32_t* scratch, cudaStream_t s, int64_t extra = 0);
+                         int32_t* pos_of, int32_t* scratch, cudaStream_t s, int32_t* zero = nullptr,
+                         int64_t extra = 0);
 
 // Plain per-galaxy forward-mode path (comparison baseline).
 size_t plain_scratch_bytes_per_row(const Consts& c);
