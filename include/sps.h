@@ -185,8 +185,8 @@ sps_status sps_create(sps_ctx** out, const sps_tables* tables, const sps_config*
 sps_status sps_destroy(sps_ctx* ctx);
 
 /* Set the galaxies (their redshifts z[n_gal], float32) that later rows refer to.
- * Computes per galaxy, in FP64 and (the wavelength sums) double-float: t_obs(z), d_L(z), the age bins in cosmic time
- * (Eq. smoothPsfh), band supports, band normalisations and AB zero points, and,
+ * Computes per galaxy, in FP64 and (the wavelength sums) double-float: t_obs(z),
+ * d_L(z), the age bins in cosmic time (Eq. smoothPsfh), band supports, band normalisations and AB zero points, and,
  * if build_approx != 0, lambda_eff (Eq. lambda_eff) and the per-galaxy table
  * c_SSP[g][b][ij] (the c_SSP definition of Sec. 3, "at a fixed z if the
  * redshift is known").  Replaces any previous set.  Synchronous. */
@@ -198,7 +198,12 @@ sps_status sps_set_galaxies(sps_ctx* ctx, const float* z, int64_t n_gal, int32_t
  * wavelength grid, dust and filters applied per wavelength); prec selects the
  * contraction arithmetic (sps_prec).  mode APPROX: Eq. photo_integral_approx
  * (FP32; prec must be SPS_FP32).  Rows whose theta is non-finite give NaN
- * magnitudes and SPS_E_NONFINITE (the other rows are still valid). */
+ * magnitudes and SPS_E_NONFINITE (the other rows are still valid).
+ * The same call on the same inputs gives the same bits.  A row's last bits may
+ * change with the number of rows in the call and, on the exact path, with the
+ * redshifts of the others, which set the tiles that its sums are split over;
+ * the tables of a galaxy and its chains in the approximate samplers do not
+ * depend on the other galaxies of the set. */
 sps_status sps_photometry(sps_ctx* ctx, const float* theta, const int32_t* gal_idx, int64_t n,
                           sps_mode mode, sps_prec prec, float* mag_out, void* stream);
 

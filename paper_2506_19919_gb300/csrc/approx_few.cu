@@ -5,8 +5,8 @@
 // chain (k_like_team and k_phot_team: one row per warp).  Here the chain is shared out:
 // each warp integrates one group of 32 age bins and takes every fourth band; the
 // sums over ages and bands meet in shared memory.
-// A call on 64 rows of six bands takes 55.5 us against 63 (photometry 45 against
-// 47), most of the rest in the host's part.
+// A call on 64 rows of six bands takes 43 us against 54 (photometry 36 against
+// 39), most of the rest in the host's part.
 #include "few.cuh"
 
 namespace sps {
@@ -255,9 +255,10 @@ k_approx_few(const __grid_constant__ Consts c, const Galaxies g, const float* __
 
 }  // namespace
 
-// Up to the rows that are resident at once (five blocks per SM): 760 rows take 54
-// us against 66 in k_like_team (photometry 44 against 51); 912 rows 64 against 66,
-// 2,432 rows 84 against 72.
+// Up to the rows that are resident at once (five blocks per SM): 760 rows take 43
+// us a call against 57 in k_like_team (photometry 37 against 41).  Past that it loses
+// its lead: 912 rows 64 against 66, 2,432 rows 84 against 72 (timed with 12 us more
+// of host work in every call).
 int64_t approx_few_rows() { return 5 * kSms; }
 
 cudaError_t launch_like_few(const Consts& c, const Galaxies& g, const float* theta, const int32_t* gal_idx, int64_t n,

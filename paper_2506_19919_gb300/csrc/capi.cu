@@ -1220,8 +1220,9 @@ extern "C" sps_status sps_hmc_run(sps_ctx* ctx, const sps_hmc_config* cfg, const
     // the first candidate is the one to beat: another replaces it only if >3% faster
     // in the probe.  One chain per warp runs 24 warps per SM in 80 registers, two
     // chains 16 in 128: 16,384 chains x 2 trajectories 9.0 ms against 11.2; two per
-    // warp stays a candidate for tables that do not fit L2, which it reads half as
-    // often, and the shape without a probe
+    // warp read the tables half as often and stay a candidate.  Without a probe the
+    // shape is still two chains per warp, with the one-chain launch for its last wave
+    // below: 300 galaxies x 16 chains 15.3 ms where one chain per warp takes 12.1
     // an age-dependent MDF runs the one-chain-per-warp variant with the per-age q matrix
     const bool rows = ctx->c.mdf_age != 0;
     std::vector<std::pair<int, int>> cands = {{1, 8}};

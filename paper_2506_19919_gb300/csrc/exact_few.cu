@@ -220,8 +220,9 @@ k_grad_few(const __grid_constant__ Consts c, const Galaxies g, const float* __re
 }  // namespace
 
 // Up to eight rows per SM: BF16 log L + gradient of six bands, a block / a warp per
-// row: 1 row 119 / 135 us a call, 100 rows 122 / 143, 608 rows 137 / 153, 1,216 rows
-// 149 / 157, 2,432 rows 189 / 185 (the rows then fill the SMs either way).
+// row: 1 row 104 / 125 us a call, 100 rows 115 / 132, 608 rows 127 / 140, 1,216 rows
+// 141 / 146; 2,432 rows 189 / 185 (timed before the forward's parts met in shared
+// memory; the rows then fill the SMs either way).
 int64_t exact_few_rows() { return 8 * kSms; }
 
 cudaError_t launch_weights_few(const Consts& c, const Grid& grid, const Galaxies& g, const float* theta,

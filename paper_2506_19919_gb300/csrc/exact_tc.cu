@@ -5,15 +5,16 @@
 //   rounding of x, and A B ~ A_hi B_hi + A_hi B_lo + A_lo B_hi (the dropped
 //   A_lo B_lo term is ~2^-22 relative), which keeps FP32-level accuracy.
 //
-// Forward: S[r][n] = sum_k W[r][k] L[k][n] for a 128-row tile and 256-wide
-// wavelength tiles, with the dust x filter reduction over n fused into the
-// epilogue (the SED never reaches HBM).  Adjoint: Wbar[r][k] = sum_n v[r][n]
-// L[k][n] for 128 x 224 tiles.
+// Forward: S[r][n] = sum_k W[r][k] L[k][n] for a 128-row tile and wavelength
+// tiles of 96 to 256 columns (fwd_shape), with the dust x filter reduction over n
+// fused into the epilogue (the SED never reaches HBM).  Adjoint: Wbar[r][k] =
+// sum_n v[r][n] L[k][n] for 128 x 224 tiles.
 //
-// Block of 6 warps, one block per SM: warp 0 issues TMA loads of A and B
-// k-blocks (128-byte rows, 128-byte swizzle) into a ring of stages; one lane
-// of warp 1 issues tcgen05.mma into one of two TMEM accumulators and commits
-// to mbarriers; warps 2-5 drain the other accumulator with tcgen05.ld.  Every
+// One block per SM: warp 0 issues TMA loads of A and B k-blocks (128-byte rows,
+// 128-byte swizzle) into a ring of stages; one lane of warp 1 issues tcgen05.mma
+// into one of two TMEM accumulators and commits to mbarriers; the other warps (8 to
+// 16 in the forward, 4 in the adjoint) drain the other accumulator with
+// tcgen05.ld.  Every
 // wait is bounded: a timeout sets the block's abort flag and the global error
 // word, the roles unwind, in-flight copies are waited for (bounded) and TMEM
 // is released.

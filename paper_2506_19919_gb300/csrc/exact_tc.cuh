@@ -31,7 +31,7 @@ constexpr int kFwdMaxEpiWarps = 16;
 // 128 registers, tiles of 192 columns (96 for 3xTF32); the epilogue is bound by
 // the latency of its exponentials and TMEM loads (100,000 rows, six bands, BF16
 // photometry 1.41 ms a call; two parts, 8 warps at 168 registers and 256 columns
-// 1.51; four parts, 16 warps at 96 registers 1.91).  Seven to 16 bands: eight per
+// 1.51; four parts, 16 warps at 96 registers 1.91; 1.28 now, with fewer spills).  Seven to 16 bands: eight per
 // warp, 8 warps at 168 registers, 256 (128) columns; more bands: eight per warp
 // in three or four groups.
 struct FwdShape {
