@@ -51,15 +51,14 @@ METRIC = "posteriors/min at fixed ESS"
 GAUSS_SIGMA_PER_FWHM = 0.42466090014400953      # 1 / (2 sqrt(2 ln 2))
 UNIT = "posteriors/min"
 
-# DRAM traffic of one bench step's k_hmc_team launches on this workload (the
-# whole waves of two-chain teams and the last wave's one-chain teams;
-# dram__bytes_read.sum + dram__bytes_write.sum, mean of five steps of a reduced
-# case with the same 4,096-galaxy working set at 50 + 50 iterations, scaled by
-# gradient evaluations to 500 + 500; profiles/k_hmc_team_hmc4096gal_x4_launches.md),
-# valid only while the kernel's sources hash to the recorded value; otherwise
-# reported as null.
+# DRAM traffic of one bench step's k_hmc_team launch on this workload (one chain
+# per warp, one launch; dram__bytes_read.sum + dram__bytes_write.sum, mean of five
+# steps of a reduced case with the same 4,096-galaxy working set at 50 + 50
+# iterations, scaled by gradient evaluations to 500 + 500;
+# profiles/k_hmc_team_hmc4096gal_x4_launches.md), valid only while the kernel's
+# sources hash to the recorded value; otherwise reported as null.
 KERNEL_SOURCES = ("hmc_team.cu", "sps_device.cuh", "sps_eval.cuh", "sps_internal.h", "philox.cuh")
-TRAFFIC = {"sha": "3c9f052df06e2568", "bytes": 217.10e9 + 11.23e9}
+TRAFFIC = {"sha": "ab086de63afd7b26", "bytes": 193.60e9 + 11.74e9}
 
 
 def _kernel_sha():
