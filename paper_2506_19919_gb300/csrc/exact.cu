@@ -252,7 +252,7 @@ k_exact_vgen(const __grid_constant__ Consts c, const Grid grid, const Galaxies g
              const float* __restrict__ theta, const int32_t* __restrict__ gal_idx, int64_t n,
              const float* __restrict__ gbar, float* __restrict__ V, uint16_t* __restrict__ Vbf,
              float* __restrict__ Vlo, const int32_t* __restrict__ perm, const uint32_t* __restrict__ hull) {
-    __shared__ float4 par[kMaxBands];       // gbar, -rest centre, inverse width (0 top-hat, < 0 table)
+    __shared__ float4 par[kMaxBands];       // gbar / kPairScale, -rest centre, inverse width (0 top-hat, < 0 table)
     __shared__ int2 sp[kMaxBands];
     const int64_t pos = blockIdx.x;
     if (pos >= n) return;
@@ -267,7 +267,7 @@ k_exact_vgen(const __grid_constant__ Consts c, const Grid grid, const Galaxies g
         const float2 ga = g.gauss[gi * B + b];
         const int kind = c.band_kind[b];
         // e^{-u^2 / 2} = 2^{-(u sqrt(log2(e) / 2))^2}
-        par[b] = make_float4(gb, -ga.x, kind == 1 ? ga.y * 0.84932180028801904f : kind == 2 ? ga.y : 0.0f, 0.0f);
+        par[b] = make_float4(gb * (1.0f / kPairScale), -ga.x, kind == 1 ? ga.y * 0.84932180028801904f : kind == 2 ? ga.y : 0.0f, 0.0f);
         const int2 s = g.support[gi * B + b];
         sp[b] = gb == 0.0f ? make_int2(0, 0) : make_int2(s.x, min(s.y, c.n_lam));
     }
@@ -286,7 +286,7 @@ k_exact_vgen(const __grid_constant__ Consts c, const Grid grid, const Galaxies g
         const int2 s = lane < B ? sp[lane] : make_int2(0, 0);
         uint32_t act = __ballot_sync(kFull, s.x < n0 + 64 && s.y > n0 && s.x < s.y);
         const float4* cp = grid.lamp + 3 * (min(nn, c.lam_pad - 2) >> 1);       // this pair's constants
-        const float4 lq = __ldg(cp);                             // lambda, q / lambda
+        const float4 lq = __ldg(cp);                             // lambda, kPairScale q / lambda
         float2 sum = make_float2(0.f, 0.f);
         for (; act; act &= act - 1) {
             const int b = __ffs(act) - 1;

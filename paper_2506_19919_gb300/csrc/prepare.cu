@@ -54,7 +54,7 @@ __device__ double drude_dshape(double lum) {
 // Per-wavelength constants: (q_n / lambda_n, k0, ln(lambda/lambda_V), Drude),
 // lambda, q / lambda, q as double-float pairs for the set-up kernels, and the
 // constants of neighbouring wavelengths side by side for packed arithmetic
-// (lamp; zero past the grid).
+// (lamp, its q / lambda times kPairScale; zero past the grid).
 __global__ void k_lambda_consts(const double* __restrict__ lam, int L, int lam_pad, float4* __restrict__ out,
                                 float* __restrict__ lam32, float4* __restrict__ lamd, float2* __restrict__ lamdq,
                                 float* __restrict__ lamp) {
@@ -74,7 +74,7 @@ __global__ void k_lambda_consts(const double* __restrict__ lam, int L, int lam_p
                          (float)drude_shape(lum));
     lam32[n] = (float)l;
     pr[0] = (float)l;
-    pr[2] = (float)(q / l);
+    pr[2] = kPairScale * (float)(q / l);
     pr[4] = out[n].y;
     pr[6] = out[n].z;
     pr[8] = out[n].w;

@@ -59,11 +59,17 @@ struct Galaxies {
     const float* dcssp;      // [G][B][K] d c_SSP / dz (approximate path) or nullptr
 };
 
+// v sums gamma_b / c_b over bands before it takes the factor q / lambda (1e-2 to
+// 1e-4): rows so faint that gamma_b / c_b nears the largest FP32 number would overflow,
+// so the sum carries 1 / kPairScale and the factor kPairScale (exact: a power of two).
+constexpr float kPairScale = 1024.0f;
+
 // Per-wavelength constants of the rest grid (device).
 struct Grid {
     const float* lam;        // [L] Angstrom
     const float4* lamc;      // [L] (q_n / lambda_n, k0, ln(lambda/lambda_V), Drude shape)
-    const float4* lamp;      // [lam_pad / 2][3] wavelength pairs: (lambda, lambda', q / lambda, q' / lambda'),
+    const float4* lamp;      // [lam_pad / 2][3] wavelength pairs: (lambda, lambda', s q / lambda, s q' / lambda'),
+                             // s = kPairScale,
                              // (k0, k0', ln(l / l_V), ln(l' / l_V)), (Drude, Drude', 0, 0)
     const double* lam64;     // [L] Angstrom, FP64
     const float4* lamd;      // [L] lambda and q_n / lambda_n as double-float pairs (hi, lo, hi, lo)
